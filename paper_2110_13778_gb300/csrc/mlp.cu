@@ -26,12 +26,14 @@ struct pb_mlp {
     cudaStream_t st = nullptr;
     float *W = nullptr, *Wm = nullptr, *Wv = nullptr, *G = nullptr;  // all weights then biases
     __nv_bfloat16* Wb = nullptr;                                      // BF16 copy of the weights
-    // training buffers (grown on demand): per layer pre-activations and BF16 activations
+    // training buffers (grown on demand): the outputs, per layer BF16 activations, dZ of two
+    // consecutive layers, and the slices of the gradient
     int cap = 0;
-    float* Z[MLP_MAXL] = {};
+    float* Z = nullptr;
     __nv_bfloat16* Ab[MLP_MAXL + 1] = {};
-    float* dA = nullptr;
-    __nv_bfloat16* dZb = nullptr;
+    __nv_bfloat16* dZb[2] = {};
+    float* part = nullptr;
+    int part_n = 0;
     float* lossbuf = nullptr;
     int* derr = nullptr;  // set by the tensor-core inference when a bounded wait gives up
     long long nparam = 0;
@@ -93,145 +95,265 @@ __device__ __forceinline__ void tc_ld32(unsigned taddr, float* v)
 }
 
 
-// ---------- generic BF16 GEMM on the fifth-generation tensor cores ----------
-// C[M x N] (FP32, ldc) = sum_k A(i, k) B(k, j) with A(i, k) = A[i * sAi + k * sAk] and
-// B(k, j) = B[k * sBk + j * sBj] (BF16, any strides; the training passes read transposed
-// operands). One block of four warps per 128 x 128 tile of C and per slice of K (gridDim.z
-// slices that add into C with atomicAdd when ksplit > 1): chunks of 64 along K are staged by
-// plain loads into shared memory in the no-swizzle K-major layout (zero outside A, B and the
-// slice), four tcgen05.mma (M = N = 128, K = 16) per chunk accumulate into 128 columns of tensor
-// memory, committed to an mbarrier; each warp then reads its 32 rows back with tcgen05.ld.
-// Every wait is bounded (a wait that gives up sets *err, waits once more and stops).
+// ---------- BF16 GEMMs of the training passes on the fifth-generation tensor cores ----------
+// C[M x N] = sum_k A(i, k) B(k, j) in FP32, one block of four warps per 128 x 128 tile of C and per
+// slice of K (blockIdx.z; slice z writes its own FP32 array, added up afterwards in slice order).
+// Every operand is stored with 8 or more consecutive elements along one index (all padded layer
+// widths are multiples of 16): along k (AK / BK: element (i, k) at [i * ld + k]) or along the
+// other index ((i, k) at [k * ld + i], the transposed operands of the gradients). A thread moves
+// 8-element (16-byte) vectors: along k straight into shared memory, otherwise eight of them
+// transposed in registers. Chunks of 64 along K go to two shared-memory stages in the no-swizzle
+// K-major layout, whose core matrices (8 rows x 16 bytes) lie GT_LBO = 144 bytes apart along k:
+// at 128 bytes the eight vectors a transposed block writes per row would all hit one bank group.
+// tcgen05.mma (M = 128, N = the tile's width rounded up to 16, K = 16) accumulates in tensor
+// memory while the next chunk is loaded; a stage is reused when the commit of its last MMAs has
+// arrived. Every wait is bounded (a wait that gives up sets *err, waits once more and stops).
+// The epilogue (one row per thread) does what used to be passes of their own:
+//   EPI_PART: FP32 tile into the slice's array; EPI_ACT: bias, ReLU, BF16 for the next layer;
+//   EPI_OUT: bias, FP32 (the output layer); EPI_MASK: the ReLU derivative, BF16 dZ.
+// What bounds these launches (4096 x 128 x 128 and smaller) is latency: one block's chain of
+// load, MMA and epilogue. Element-by-element staging through 2-byte loads and K slices of 2048
+// took 128 us per launch: a mini-batch's gradient (4096 rows, 18-128-128-128-2, to the host) takes
+// 215 us now, 1469 us then.
 #define GT_K 64
-__device__ __forceinline__ unsigned gt_off(int r, int k) { return (r >> 3) * (GT_K / 8) * 128 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2; }
-__device__ __forceinline__ unsigned gt_su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+#define GT_LBO 144
+#define GT_SBO ((GT_K / 8) * GT_LBO)
+#define GT_STAGE (16 * GT_SBO)  // bytes of one operand's stage: 128 rows
+#define GT_SMEM (4 * GT_STAGE)
+enum { EPI_PART, EPI_ACT, EPI_OUT, EPI_MASK };
+__device__ __forceinline__ unsigned gt_off(int r, int k8) { return (r >> 3) * GT_SBO + k8 * GT_LBO + (r & 7) * 16; }
 
-__global__ void __launch_bounds__(128, 1) k_gemm_tc(int M, int N, int K, const __nv_bfloat16* __restrict__ A,
-                                                    long long sAi, long long sAk, const __nv_bfloat16* __restrict__ B,
-                                                    long long sBk, long long sBj, float* __restrict__ C, long long ldc,
-                                                    int accumulate, int* __restrict__ err)
+// rows [r0, r0 + 128) (fewer than R: zeros), k in [k0, ke) of an operand stored along k
+__device__ __forceinline__ void gt_stage_k(unsigned char* sm, const __nv_bfloat16* __restrict__ X, long long ld, int r0,
+                                           int R, int k0, int ke, int rows)
 {
-    __shared__ __align__(128) __nv_bfloat16 As[128 * GT_K], Bs[128 * GT_K];
-    __shared__ __align__(8) unsigned long long bar;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        const int e = threadIdx.x + 128 * v;  // 8 rows x 8 vectors per 64 threads: rows fastest
+        const int r = (e >> 6) * 8 + (e & 7), k8 = (e >> 3) & 7;
+        const int k = k0 + 8 * k8;
+        if (r >= rows) continue;
+        uint4 w = make_uint4(0, 0, 0, 0);
+        if (r0 + r < R && k < ke) w = *reinterpret_cast<const uint4*>(X + (long long)(r0 + r) * ld + k);
+        *reinterpret_cast<uint4*>(sm + gt_off(r, k8)) = w;
+    }
+}
+// the same of an operand stored along its rows: 8 x 8 blocks, transposed; R is a multiple of 8.
+// SUM: adds the block's eight k into cs[8] (the column sums that are the bias gradient)
+template <bool SUM>
+__device__ __forceinline__ void gt_stage_r(unsigned char* sm, const __nv_bfloat16* __restrict__ X, long long ld, int r0,
+                                           int R, int k0, int ke, int rows, float* cs)
+{
+    const int rb = threadIdx.x & 15, k8 = threadIdx.x >> 4;  // rows fastest: coalesced loads
+    if (8 * rb >= rows) return;
+    uint4 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int k = k0 + 8 * k8 + q;
+        v[q] = make_uint4(0, 0, 0, 0);
+        if (r0 + 8 * rb < R && k < ke) v[q] = *reinterpret_cast<const uint4*>(X + (long long)k * ld + r0 + 8 * rb);
+    }
+    if (SUM) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const unsigned w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                cs[2 * c] += __uint_as_float(w[c] << 16);
+                cs[2 * c + 1] += __uint_as_float(w[c] & 0xffff0000u);
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        unsigned w[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q] = c == 0 ? v[q].x : c == 1 ? v[q].y : c == 2 ? v[q].z : v[q].w;
+        *reinterpret_cast<uint4*>(sm + gt_off(8 * rb + 2 * c, k8)) =
+            make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410),
+                       __byte_perm(w[4], w[5], 0x5410), __byte_perm(w[6], w[7], 0x5410));
+        *reinterpret_cast<uint4*>(sm + gt_off(8 * rb + 2 * c + 1, k8)) =
+            make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632),
+                       __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
+    }
+}
+
+struct GemmArgs {
+    int M, N, K;
+    const __nv_bfloat16 *A, *B;
+    long long lda, ldb;
+    float* C;                   // EPI_PART, EPI_OUT: FP32 result (row stride N; slice z at + z * cstr)
+    long long cstr;
+    __nv_bfloat16* Cb;          // EPI_ACT, EPI_MASK: BF16 result (row stride N)
+    const float* bias;          // EPI_ACT, EPI_OUT
+    const __nv_bfloat16* mask;  // EPI_MASK: the activations whose positive entries pass
+    float* csum;                // EPI_PART: column sums of A over k (the bias gradient), slice z at + z * cstr
+    int kslice;                 // multiple of GT_K
+};
+
+template <bool AK, bool BK, int EPI>
+__global__ void __launch_bounds__(128) k_gemm_tc(GemmArgs g, int* __restrict__ err)
+{
+    extern __shared__ __align__(128) unsigned char gsm[];
+    __shared__ __align__(8) unsigned long long bar[2];
     __shared__ unsigned tslot;
+    __shared__ float csh[EPI == EPI_PART ? 8 : 1][EPI == EPI_PART ? 128 : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int i0 = blockIdx.x * 128, j0 = blockIdx.y * 128;
-    const int kslice = (K + gridDim.z - 1) / gridDim.z;
-    const int kb = blockIdx.z * kslice, ke = min(K, kb + kslice);
+    const int kb = blockIdx.z * g.kslice, ke = min(g.K, kb + g.kslice);
+    const int nn = min(128, ((g.N - j0) + 15) & ~15);  // columns of this tile (a multiple of 16)
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(gt_su32(&bar)) : "memory");
+        for (int b = 0; b < 2; ++b)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_su32(&bar[b])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(gt_su32(&tslot)),
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_su32(&tslot)),
                      "r"(128)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const unsigned taddr = tslot;
-    const unsigned idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-    const unsigned sbo = (GT_K / 8) * 128;
-    const __nv_bfloat16 z = __float2bfloat16(0.f);
-    unsigned ph = 0u;
-    bool alive = true, any = false;
-    for (int k0 = kb; k0 < ke && alive; k0 += GT_K) {
-        for (int e = tid; e < 128 * GT_K; e += 128) {
-            const int r = e / GT_K, kk = e % GT_K, k = k0 + kk;
-            const int i = i0 + r, j = j0 + r;
-            const bool kin = k < ke;
-            *(__nv_bfloat16*)((char*)As + gt_off(r, kk)) = (kin && i < M) ? A[(long long)i * sAi + (long long)k * sAk] : z;
-            *(__nv_bfloat16*)((char*)Bs + gt_off(r, kk)) = (kin && j < N) ? B[(long long)k * sBk + (long long)j * sBj] : z;
+    tc_fence_after();
+    const unsigned taddr = tslot, idesc = tc_idesc(nn);
+    float cs[8] = {};
+    unsigned ph[2] = {0u, 0u};
+    bool alive = true;
+    int c = 0;
+    for (int k0 = kb; k0 < ke; k0 += GT_K, ++c) {
+        const int b = c & 1;
+        unsigned char *As = gsm + b * 2 * GT_STAGE, *Bs = As + GT_STAGE;
+        if (c >= 2) {  // the MMAs that read this stage two chunks ago are done
+            if (!__syncthreads_and(tc_wait(tc_su32(&bar[b]), ph[b]))) {
+                if (tid == 0) atomicExch(err, 1);
+                tc_wait(tc_su32(&bar[b]), ph[b]);  // let the MMAs in flight finish before the memory goes
+                tc_wait(tc_su32(&bar[b ^ 1]), ph[b ^ 1]);
+                alive = false;
+                break;
+            }
+            ph[b] ^= 1u;
         }
+        if (AK) gt_stage_k(As, g.A, g.lda, i0, g.M, k0, ke, 128);
+        else gt_stage_r<EPI == EPI_PART>(As, g.A, g.lda, i0, g.M, k0, ke, 128, cs);
+        if (BK) gt_stage_k(Bs, g.B, g.ldb, j0, g.N, k0, ke, nn);
+        else gt_stage_r<false>(Bs, g.B, g.ldb, j0, g.N, k0, ke, nn, cs);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        tc_fence_before();
         __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tc_fence_after();
         if (tid == 0) {
-            for (int ks = 0; ks < GT_K / 16; ++ks) {
-                const uint64_t ad = tc_desc(gt_su32(As) + ks * 256, 128, sbo);
-                const uint64_t bd = tc_desc(gt_su32(Bs) + ks * 256, 128, sbo);
+            const int steps = (min(GT_K, ke - k0) + 15) / 16;
+            for (int ks = 0; ks < steps; ++ks) {
+                const uint64_t ad = tc_desc(tc_su32(As) + ks * 2 * GT_LBO, GT_LBO, GT_SBO);
+                const uint64_t bd = tc_desc(tc_su32(Bs) + ks * 2 * GT_LBO, GT_LBO, GT_SBO);
                 asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                             ::"r"(taddr), "l"(ad), "l"(bd), "r"(idesc), "r"((unsigned)(any || ks > 0)) : "memory");
+                             ::"r"(taddr), "l"(ad), "l"(bd), "r"(idesc), "r"((unsigned)(c > 0 || ks > 0)) : "memory");
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         ::"r"(gt_su32(&bar)) : "memory");
+                         ::"r"(tc_su32(&bar[b])) : "memory");
         }
-        any = true;
-        if (!__syncthreads_and(tc_wait(gt_su32(&bar), ph))) {
-            if (tid == 0) atomicExch(err, 1);
-            tc_wait(gt_su32(&bar), ph);
-            alive = false;
-            break;
-        }
-        ph ^= 1u;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
-    if (alive && (any || !accumulate)) {
-        const int i = i0 + 32 * warp + lane;
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-            float v[32];
-            if (any) tc_ld32(taddr + ((unsigned)(32 * warp) << 16) + c0, v);
-            else
-                for (int q = 0; q < 32; ++q) v[q] = 0.f;
-            if (i < M)
-                for (int q = 0; q < 32; ++q) {
-                    const int j = j0 + c0 + q;
-                    if (j < N) {
-                        float* c = C + (long long)i * ldc + j;
-                        if (accumulate) atomicAdd(c, v[q]);
-                        else *c = v[q];
+    // the outstanding commits (the last two chunks')
+    for (int d = max(0, c - 2); d < c && alive; ++d) {
+        const int b = d & 1;
+        if (!__syncthreads_and(tc_wait(tc_su32(&bar[b]), ph[b]))) {
+            if (tid == 0) atomicExch(err, 1);
+            tc_wait(tc_su32(&bar[b]), ph[b]);
+            alive = false;
+        }
+        ph[b] ^= 1u;
+    }
+    tc_fence_after();
+    const int i = i0 + 32 * warp + lane;
+    for (int c0 = 0; c0 < nn && alive; c0 += 32) {
+        float v[32];
+        __syncwarp();
+        if (c > 0) tc_ld32(taddr + ((unsigned)(32 * warp) << 16) + c0, v);  // (columns past nn are not used)
+        else
+            for (int q = 0; q < 32; ++q) v[q] = 0.f;
+        if (i >= g.M) continue;
+        const int w = min(32, nn - c0);  // 16 or 32
+#pragma unroll
+        for (int q = 0; q < 32; q += 8) {
+            if (q >= w) break;
+            const int j = j0 + c0 + q;
+            const long long o = (long long)i * g.N + j;
+            if (EPI == EPI_PART || EPI == EPI_OUT) {
+                float* dst = g.C + (EPI == EPI_PART ? blockIdx.z * g.cstr : 0) + o;
+#pragma unroll
+                for (int h = 0; h < 8; h += 4) {
+                    float4 f = make_float4(v[q + h], v[q + h + 1], v[q + h + 2], v[q + h + 3]);
+                    if (EPI == EPI_OUT) {
+                        const float* bi = g.bias + j + h;
+                        f = make_float4(f.x + bi[0], f.y + bi[1], f.z + bi[2], f.w + bi[3]);
+                    }
+                    *reinterpret_cast<float4*>(dst + h) = f;
+                }
+            } else {
+                __align__(16) __nv_bfloat16 r[8];
+                if (EPI == EPI_ACT) {
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) r[h] = __float2bfloat16(fmaxf(v[q + h] + g.bias[j + h], 0.f));
+                } else {
+                    const uint4 mk = *reinterpret_cast<const uint4*>(g.mask + o);
+                    const unsigned mw[4] = {mk.x, mk.y, mk.z, mk.w};
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) {
+                        const float a = __uint_as_float(h & 1 ? mw[h >> 1] & 0xffff0000u : mw[h >> 1] << 16);
+                        r[h] = __float2bfloat16(a > 0.f ? v[q + h] : 0.f);
                     }
                 }
+                *reinterpret_cast<uint4*>(g.Cb + o) = *reinterpret_cast<const uint4*>(r);
+            }
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (EPI == EPI_PART && alive && blockIdx.y == 0) {  // column sums: the threads' k groups in order
+#pragma unroll
+        for (int q = 0; q < 8; ++q) csh[tid >> 4][(tid & 15) * 8 + q] = cs[q];
+        __syncthreads();
+        float s = 0.f;
+        for (int q = 0; q < 8; ++q) s += csh[q][tid];
+        if (i0 + tid < g.M) g.csum[blockIdx.z * g.cstr + i0 + tid] = s;
+    }
+    tc_fence_before();
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(128) : "memory");
 }
 
-static void gemm(cudaStream_t st, int M, int N, int K, const __nv_bfloat16* A, long long sAi, long long sAk,
-                 const __nv_bfloat16* B, long long sBk, long long sBj, float* C, long long ldc, int ksplit, int* err)
+template <bool AK, bool BK, int EPI>
+static bool gemm(cudaStream_t st, GemmArgs g, int slices, int* err)
 {
-    dim3 grid((M + 127) / 128, (N + 127) / 128, ksplit);
-    k_gemm_tc<<<grid, 128, 0, st>>>(M, N, K, A, sAi, sAk, B, sBk, sBj, C, ldc, ksplit > 1, err);
+    if (cudaFuncSetAttribute(k_gemm_tc<AK, BK, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, GT_SMEM) !=
+        cudaSuccess)
+        return false;
+    const int per = (g.K + slices - 1) / slices;
+    g.kslice = (per + GT_K - 1) / GT_K * GT_K;
+    const dim3 grid((g.M + 127) / 128, (g.N + 127) / 128, slices);
+    k_gemm_tc<AK, BK, EPI><<<grid, 128, GT_SMEM, st>>>(g, err);
+    return true;
 }
 
 // ---------- elementwise pieces ----------
-__global__ void k_to_bf16(long long n, const float* __restrict__ x, __nv_bfloat16* __restrict__ y)
+// Before a training pass: the weights as BF16, the input rows (n x nin, FP32) as a zero-padded
+// BF16 matrix (n x dpad), and a zero loss
+__global__ void k_prepare(long long nw, const float* __restrict__ w, __nv_bfloat16* __restrict__ wb, int n, int nin,
+                          int dpad, const float* __restrict__ X, __nv_bfloat16* __restrict__ Y, float* __restrict__ loss)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16(x[i]);
-}
-
-// input rows (n x nin, FP32) into a zero-padded BF16 matrix (n x dpad)
-__global__ void k_pack_input(int n, int nin, int dpad, const float* __restrict__ X, __nv_bfloat16* __restrict__ Y)
-{
-    long long tot = (long long)n * dpad;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
+    const long long tot = (long long)n * dpad, stride = (long long)gridDim.x * blockDim.x;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *loss = 0.f;
+    for (long long i = t; i < nw; i += stride) wb[i] = __float2bfloat16(w[i]);
+    for (long long i = t; i < tot; i += stride) {
         int r = (int)(i / dpad), c = (int)(i % dpad);
         Y[i] = __float2bfloat16(c < nin ? X[(long long)r * nin + c] : 0.f);
     }
 }
 
-// Z += bias; A = relu(Z) (hidden) or Z (output), as BF16 for the next layer
-__global__ void k_bias_act(int n, int d, const float* __restrict__ b, float* __restrict__ Z,
-                           __nv_bfloat16* __restrict__ Ab, int relu)
-{
-    long long tot = (long long)n * d;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
-        float v = Z[i] + b[i % d];
-        Z[i] = v;
-        if (Ab) Ab[i] = __float2bfloat16(relu ? fmaxf(v, 0.f) : v);
-    }
-}
-
-// output layer: dZ = 2 (Y - T) / (n nout) on the real outputs, loss partial sums
+// output layer: dZ = 2 (Y - T) / (n nout) on the real outputs (BF16), loss partial sums
 __global__ void k_mse(int n, int nout, int dpad, const float* __restrict__ Y, const float* __restrict__ T,
-                      float* __restrict__ dZ, float* __restrict__ loss)
+                      __nv_bfloat16* __restrict__ dZ, float* __restrict__ loss)
 {
     __shared__ float red[256];
     float s = 0.f;
@@ -245,7 +367,7 @@ __global__ void k_mse(int n, int nout, int dpad, const float* __restrict__ Y, co
             s += e * e;
             g = sc * e;
         }
-        dZ[i] = g;
+        dZ[i] = __float2bfloat16(g);
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -256,28 +378,15 @@ __global__ void k_mse(int n, int nout, int dpad, const float* __restrict__ Y, co
     if (threadIdx.x == 0) atomicAdd(loss, red[0] / ((float)n * (float)nout));
 }
 
-// dZ = dA * relu'(Z)
-__global__ void k_relu_back(long long n, const float* __restrict__ Z, const float* __restrict__ dA,
-                            __nv_bfloat16* __restrict__ dZb)
+// the gradient: the slices' parts added in slice order (results do not depend on scheduling)
+__global__ void k_sum_slices(long long n, int slices, const float* __restrict__ part, float* __restrict__ out)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dZb[i] = __float2bfloat16(Z[i] > 0.f ? dA[i] : 0.f);
-}
-
-// bias gradient: column sums of dZ (n x d)
-__global__ void k_colsum(int n, int d, const __nv_bfloat16* __restrict__ dZ, float* __restrict__ gb)
-{
-    int c = blockIdx.x;
-    float s = 0.f;
-    for (int r = threadIdx.x; r < n; r += blockDim.x) s += __bfloat162float(dZ[(long long)r * d + c]);
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        float s = 0.f;
+#pragma unroll 8
+        for (int z = 0; z < slices; ++z) s += part[z * n + i];
+        out[i] = s;
     }
-    if (threadIdx.x == 0) gb[c] = red[0];
 }
 
 __global__ void k_adam(long long n, float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
@@ -308,29 +417,35 @@ __global__ void k_init(long long n, float* __restrict__ w, float s, unsigned lon
 
 static int grid1(long long n) { return (int)std::min<long long>((n + 255) / 256, 152 * 8); }
 
+// slices of the rows that a weight gradient sums over: of 128 rows or more (at 4096 rows 32 blocks
+// per gradient; 2 slices of 2048 rows took 128 us each), at most 64, and at most 64 MB of parts
+// (a wide network's gradients have tiles enough)
+static int grad_slices(const pb_mlp* m, int n)
+{
+    const long long most = std::max(1LL, std::min(64LL, (16LL << 20) / m->nparam));
+    return (int)std::max(1LL, std::min(most, (long long)n / 128));
+}
+
 static int ensure_cap(pb_mlp* m, int n)
 {
     if (n <= m->cap) return PB_OK;
     cudaStreamSynchronize(m->st);
-    for (int l = 0; l < m->nl; ++l) {
-        cudaFree(m->Z[l]);
-        m->Z[l] = nullptr;
-    }
+    cudaFree(m->Z);
+    m->Z = nullptr;
     for (int l = 0; l <= m->nl; ++l) {
         cudaFree(m->Ab[l]);
         m->Ab[l] = nullptr;
     }
-    cudaFree(m->dA);
-    cudaFree(m->dZb);
     int dmax = 16;
     for (int l = 0; l < m->nl; ++l) dmax = std::max(dmax, std::max(m->din[l], m->dout[l]));
-    bool ok = true;
-    for (int l = 0; l < m->nl; ++l) ok &= cudaMalloc(&m->Z[l], sizeof(float) * (size_t)n * m->dout[l]) == cudaSuccess;
-    ok &= cudaMalloc(&m->Ab[0], sizeof(__nv_bfloat16) * (size_t)n * m->din[0]) == cudaSuccess;
+    for (auto& d : m->dZb) {
+        cudaFree(d);
+        d = nullptr;
+    }
+    bool ok = cudaMalloc(&m->Z, sizeof(float) * (size_t)n * m->dout[m->nl - 1]) == cudaSuccess;
     for (int l = 0; l < m->nl; ++l)
-        ok &= cudaMalloc(&m->Ab[l + 1], sizeof(__nv_bfloat16) * (size_t)n * m->dout[l]) == cudaSuccess;
-    ok &= cudaMalloc(&m->dA, sizeof(float) * (size_t)n * dmax) == cudaSuccess;
-    ok &= cudaMalloc(&m->dZb, sizeof(__nv_bfloat16) * (size_t)n * dmax) == cudaSuccess;
+        ok &= cudaMalloc(&m->Ab[l], sizeof(__nv_bfloat16) * (size_t)n * m->din[l]) == cudaSuccess;
+    for (auto& d : m->dZb) ok &= cudaMalloc(&d, sizeof(__nv_bfloat16) * (size_t)n * dmax) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         m->cap = 0;
@@ -340,45 +455,74 @@ static int ensure_cap(pb_mlp* m, int n)
     return PB_OK;
 }
 
-// forward pass over n rows; keeps Z and BF16 activations for a backward pass
+// the gradient's slices (only a backward pass needs them)
+static int ensure_part(pb_mlp* m, int slices)
+{
+    if (slices <= m->part_n) return PB_OK;
+    cudaStreamSynchronize(m->st);
+    cudaFree(m->part);
+    m->part = nullptr;
+    m->part_n = 0;
+    if (cudaMalloc(&m->part, sizeof(float) * (size_t)m->nparam * slices) != cudaSuccess) {
+        cudaGetLastError();
+        return mlp_fail(m, PB_ERR_NOMEM, "mlp: out of memory");
+    }
+    m->part_n = slices;
+    return PB_OK;
+}
+
+// forward pass over n rows; keeps the outputs and the BF16 activations for a backward pass
 static int mlp_forward(pb_mlp* m, const float* X, int n)
 {
     int rc = ensure_cap(m, n);
     if (rc) return rc;
-    k_to_bf16<<<grid1(m->nparam), 256, 0, m->st>>>(m->nparam, m->W, m->Wb);
-    k_pack_input<<<grid1((long long)n * m->din[0]), 256, 0, m->st>>>(n, m->nin, m->din[0], X, m->Ab[0]);
+    const long long most = std::max(m->nparam, (long long)n * m->din[0]);
+    k_prepare<<<grid1(most), 256, 0, m->st>>>(m->nparam, m->W, m->Wb, n, m->nin, m->din[0], X, m->Ab[0], m->lossbuf);
+    bool ok = true;
     for (int l = 0; l < m->nl; ++l) {
-        const int k = m->din[l], d = m->dout[l];
         // Z = A W^T: B(kk, j) = W[j][kk]
-        gemm(m->st, n, d, k, m->Ab[l], k, 1, m->Wb + m->woff[l], 1, k, m->Z[l], d, 1, m->derr);
-        k_bias_act<<<grid1((long long)n * d), 256, 0, m->st>>>(n, d, m->W + m->boff[l], m->Z[l], m->Ab[l + 1],
-                                                               l + 1 < m->nl);
+        GemmArgs g = {n, m->dout[l], m->din[l], m->Ab[l], m->Wb + m->woff[l], m->din[l], m->din[l]};
+        g.bias = m->W + m->boff[l];
+        if (l + 1 < m->nl) {
+            g.Cb = m->Ab[l + 1];
+            ok &= gemm<true, true, EPI_ACT>(m->st, g, 1, m->derr);
+        } else {
+            g.C = m->Z;
+            ok &= gemm<true, true, EPI_OUT>(m->st, g, 1, m->derr);
+        }
     }
-    return cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp forward launch failed");
+    return ok && cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp forward launch failed");
 }
 
 // backward pass after mlp_forward: gradients into m->G, loss into m->lossbuf
 static int mlp_backward(pb_mlp* m, const float* T, int n)
 {
-    const int L = m->nl;
-    cudaMemsetAsync(m->G, 0, sizeof(float) * m->nparam, m->st);
-    cudaMemsetAsync(m->lossbuf, 0, sizeof(float), m->st);
+    const int L = m->nl, slices = grad_slices(m, n);
+    int rc = ensure_part(m, slices);
+    if (rc) return rc;
     const int dl = m->dout[L - 1];
-    k_mse<<<grid1((long long)n * dl), 256, 0, m->st>>>(n, m->nout, dl, m->Z[L - 1], T, m->dA, m->lossbuf);
-    k_to_bf16<<<grid1((long long)n * dl), 256, 0, m->st>>>((long long)n * dl, m->dA, m->dZb);
-    for (int l = L - 1; l >= 0; --l) {
+    k_mse<<<grid1((long long)n * dl), 256, 0, m->st>>>(n, m->nout, dl, m->Z, T, m->dZb[0], m->lossbuf);
+    bool ok = true;
+    int cur = 0;
+    for (int l = L - 1; l >= 0; --l, cur ^= 1) {
         const int k = m->din[l], d = m->dout[l];
-        // dW = dZ^T A: A-operand (i = out unit, kk = row) = dZ[kk][i]; B(kk = row, j = in) = A[kk][j]
-        const int ks = std::max(1, std::min(64, n / 2048));
-        gemm(m->st, d, k, n, m->dZb, 1, d, m->Ab[l], k, 1, m->G + m->woff[l], k, ks, m->derr);
-        k_colsum<<<d, 256, 0, m->st>>>(n, d, m->dZb, m->G + m->boff[l]);
+        // dW = dZ^T A: A-operand (i = out unit, kk = row) = dZ[kk][i]; B(kk = row, j = in) = A[kk][j];
+        // db = the column sums of dZ
+        GemmArgs w = {d, k, n, m->dZb[cur], m->Ab[l], d, k};
+        w.C = m->part + m->woff[l];
+        w.csum = m->part + m->boff[l];
+        w.cstr = m->nparam;
+        ok &= gemm<false, false, EPI_PART>(m->st, w, slices, m->derr);
         if (l > 0) {
-            // dA_prev = dZ W: A(i = row, kk = out) = dZ[i][kk]; B(kk = out, j = in) = W[kk][j]
-            gemm(m->st, n, k, d, m->dZb, d, 1, m->Wb + m->woff[l], k, 1, m->dA, k, 1, m->derr);
-            k_relu_back<<<grid1((long long)n * k), 256, 0, m->st>>>((long long)n * k, m->Z[l - 1], m->dA, m->dZb);
+            // dZ_prev = relu'(Z_prev) (dZ W): A(i = row, kk = out) = dZ[i][kk]; B(kk = out, j = in) = W[kk][j]
+            GemmArgs g = {n, k, d, m->dZb[cur], m->Wb + m->woff[l], d, k};
+            g.Cb = m->dZb[cur ^ 1];
+            g.mask = m->Ab[l];
+            ok &= gemm<true, false, EPI_MASK>(m->st, g, 1, m->derr);
         }
     }
-    return cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp backward launch failed");
+    k_sum_slices<<<grid1(m->nparam), 256, 0, m->st>>>(m->nparam, slices, m->part, m->G);
+    return ok && cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp backward launch failed");
 }
 
 extern "C" int pb_mlp_create(int nin, int width, int depth, int nout, unsigned long long seed, void* stream,
@@ -460,10 +604,10 @@ extern "C" int pb_mlp_destroy(pb_mlp* m)
     cudaFree(m->Wb);
     cudaFree(m->lossbuf);
     cudaFree(m->derr);
-    for (int l = 0; l < MLP_MAXL; ++l) cudaFree(m->Z[l]);
+    cudaFree(m->Z);
     for (int l = 0; l <= MLP_MAXL; ++l) cudaFree(m->Ab[l]);
-    cudaFree(m->dA);
-    cudaFree(m->dZb);
+    for (auto& d : m->dZb) cudaFree(d);
+    cudaFree(m->part);
     delete m;
     return PB_OK;
 }
@@ -676,7 +820,7 @@ extern "C" int pb_mlp_forward(pb_mlp* m, const float* X, int n, float* Y)
     if (rc) return rc;
     // real outputs of the last layer, row-major n x nout
     const int L = m->nl, dl = m->dout[L - 1];
-    if (cudaMemcpy2DAsync(Y, sizeof(float) * m->nout, m->Z[L - 1], sizeof(float) * dl, sizeof(float) * m->nout, n,
+    if (cudaMemcpy2DAsync(Y, sizeof(float) * m->nout, m->Z, sizeof(float) * dl, sizeof(float) * m->nout, n,
                           cudaMemcpyDeviceToDevice, m->st) != cudaSuccess)
         return mlp_fail(m, PB_ERR_CUDA, "mlp: output copy failed");
     return PB_OK;

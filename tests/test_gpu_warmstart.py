@@ -107,6 +107,28 @@ def test_gradient_matches_oracle(net, n):
     assert np.all(G[0][0][:, 18:] == 0) and np.all(G[-1][0][2:, :] == 0) and np.all(G[-1][1][2:] == 0)
 
 
+@pytest.mark.parametrize("shape,n", [((18, 128, 3, 2), 127), ((18, 128, 3, 2), 129), ((18, 128, 3, 2), 4097),
+                                     ((5, 64, 2, 3), 300), ((40, 256, 1, 33), 1000), ((16, 144, 2, 17), 513)])
+def test_gradient_tiles_and_row_slices(shape, n):
+    # one row slice and several, with remainders; tiles of 16 to 128 columns and two tiles per
+    # matrix; the same bfloat16 rounding points as the oracle's emulation (bar: 2e-2 as above)
+    h = pb.pb_mlp_create(*shape, seed=5)
+    try:
+        w = omlp.init_params(shape, 6).astype(np.float32)
+        pb.pb_mlp_set_params(h, w)
+        rng = np.random.default_rng(n)
+        X = rng.standard_normal((n, shape[0])).astype(np.float32)
+        T = rng.standard_normal((n, shape[3])).astype(np.float32)
+        loss, g = pb.pb_mlp_gradient(h, torch.from_numpy(X).cuda(), torch.from_numpy(T).cuda())
+        lo, go = omlp.loss_grad(w.astype(np.float64), shape, X.astype(np.float64), T.astype(np.float64), emulate=True)
+        assert abs(loss - lo) < 1e-3 * lo
+        for (gw, gb), (ow, ob) in zip(omlp.unpack(g.astype(np.float64), shape), omlp.unpack(go, shape)):
+            assert _rel(gw, ow) < 2e-2
+            assert _rel(gb, ob) < 2e-2
+    finally:
+        pb.pb_mlp_destroy(h)
+
+
 def test_adam_step_matches_oracle(net):
     w = omlp.init_params(SHAPE, 3).astype(np.float32)
     pb.pb_mlp_set_params(net, w)
