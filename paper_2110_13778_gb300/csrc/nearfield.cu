@@ -9,9 +9,8 @@
 //   y1_i = 1/2 (1 + eps) A_i phi_i     - sum_j (I1_ij dphi_j + I2_ij phi_j)
 //   y2_i = 1/2 (1 + 1/eps) A_i dphi_i  - sum_j (I3_ij dphi_j + I4_ij phi_j)
 //
-// Layout (FP64): one CTA per target leaf, one thread per target element. Source leaves are
-// staged tile by tile in shared memory (centroid, area, normal, A_j phi_j, A_j dphi_j) and read
-// as warp-wide broadcasts. Mixed precision: one warp per chunk of up to 32 targets, which
+// Layout: both precisions work on pair tiles of chunks of at most 32 elements of neighbouring
+// leaves (FP64: k_near64). Mixed precision: one warp per chunk of up to 32 targets, which
 // evaluates each pair of distinct chunks once for both directions (k_near_tile; several
 // right-hand sides: k_near32m, one direction, up to 16 densities per pair evaluation). In
 // mixed precision each source leaf's partial sums are kept in FP32
@@ -27,95 +26,199 @@
 #include "pb_internal.cuh"
 
 
-#define NEAR_T 128
 #define NEAR_ITEM 6    // pair tiles per warp of the mixed-precision near field
 #define NEAR_ITEM_M 8  // directed tiles per warp of the several-vector near field
 
-template <class R, class PV, bool HILO>
-__global__ void __launch_bounds__(NEAR_T) k_near(int nt, const int* __restrict__ begin,
-                                                 const int* __restrict__ noff, const int* __restrict__ nidx,
-                                                 const PV* __restrict__ ep, const PV* __restrict__ en,
-                                                 const float4* __restrict__ elo, const double* __restrict__ xs,
-                                                 double eps_d, double kappa_d, double* __restrict__ ys)
+// ---------- FP64 near field ----------
+// Pair tiles as in the mixed-precision kernel below: one warp per pair of chunks (A, B) of at most
+// 32 elements of neighbouring leaves evaluates each pair once for both directions. The FP64 pipe
+// (1/64 of the FP32 rate) is all that counts here: 53 FP64 operations, one reciprocal square root
+// and one exponential per pair of elements, where one direction at a time took 45 and the same
+// two functions per direction. The larger chunk goes to the lanes and the other is walked, so
+// that only the steps of a remainder chunk with a remainder chunk leave lanes idle. At step s
+// lane l meets source (l mod nb + s) mod nb; the sources' sums live in shared memory, one set
+// per group of nb lanes, so that the lanes of a step write different words and the sum of a
+// source has a fixed order. Every tile writes the sums of both its chunks (2 x 2 x 32 doubles),
+// which k_near64_sum adds per element in tile order: no atomics, and the product does not depend
+// on scheduling. 20,480 elements: near field 1.80 ms; 11.3 ms one direction at a time with a block of 128
+// threads per leaf of 76.
+struct Near64Src {
+    double x[32], y[32], z[32], nx[32], ny[32], nz[32], phi[32], dphi[32];
+    double r1[64], r2[64];  // ceil(32 / nb) groups of nb <= 32 sums: at most 63
+};
+__global__ void __launch_bounds__(256, 2) k_near64(int nt, int ntiles, const int2* __restrict__ tiles,
+                                                const int* __restrict__ chunk_leaf,
+                                                const int* __restrict__ chunk_first, const int* __restrict__ begin,
+                                                const double4_32a* __restrict__ ep, const double4_32a* __restrict__ en,
+                                                const double* __restrict__ xs, double eps, double kappa,
+                                                double* __restrict__ part)
 {
-    __shared__ R sx[NEAR_T], sy[NEAR_T], sz[NEAR_T], snx[NEAR_T], sny[NEAR_T], snz[NEAR_T];
-    __shared__ R sphi[NEAR_T], sdphi[NEAR_T];
-    __shared__ R slx[HILO ? NEAR_T : 1], sly[HILO ? NEAR_T : 1], slz[HILO ? NEAR_T : 1];
-    const int c = blockIdx.x;
-    const int tb = begin[c], te = begin[c + 1];
-    const R eps = (R)eps_d, inv_eps = (R)(1.0 / eps_d), kappa = (R)kappa_d;
-    for (int t0 = tb; t0 < te; t0 += NEAR_T) {
-        const int k = t0 + threadIdx.x;
-        const bool act = k < te;
-        R px = 0, py = 0, pz = 0, qx = 0, qy = 0, qz = 0, lx = 0, ly = 0, lz = 0;
-        if (act) {
-            PV p = ep[k], n = en[k];
-            if (HILO) {
-                float4 l = elo[k];
-                lx = l.x;
-                ly = l.y;
-                lz = l.z;
-            }
-            px = (R)p.x;
-            py = (R)p.y;
-            pz = (R)p.z;
-            qx = (R)n.x;
-            qy = (R)n.y;
-            qz = (R)n.z;
-        }
-        double acc1 = 0.0, acc2 = 0.0;
-        for (int t = noff[c]; t < noff[c + 1]; ++t) {
-            const int c2 = nidx[t];
-            const int sb = begin[c2], se = begin[c2 + 1];
-            R s1 = 0, s2 = 0;
-            for (int s0 = sb; s0 < se; s0 += NEAR_T) {
-                const int ns = min(NEAR_T, se - s0);
-                __syncthreads();
-                if (threadIdx.x < ns) {
-                    const int j = s0 + threadIdx.x;
-                    PV p = ep[j], n = en[j];
-                    sx[threadIdx.x] = (R)p.x;
-                    sy[threadIdx.x] = (R)p.y;
-                    sz[threadIdx.x] = (R)p.z;
-                    snx[threadIdx.x] = (R)n.x;
-                    sny[threadIdx.x] = (R)n.y;
-                    snz[threadIdx.x] = (R)n.z;
-                    sphi[threadIdx.x] = (R)(p.w * xs[j]);
-                    sdphi[threadIdx.x] = (R)(p.w * xs[nt + j]);
-                    if (HILO) {
-                        float4 l = elo[j];
-                        slx[threadIdx.x] = l.x;
-                        sly[threadIdx.x] = l.y;
-                        slz[threadIdx.x] = l.z;
-                    }
-                }
-                __syncthreads();
-                if (act) {
-#pragma unroll 4
-                    for (int q = 0; q < ns; ++q) {
-                        if (s0 + q == k) continue;
-                        R K[4];
-                        R dx = px - sx[q], dy = py - sy[q], dz = pz - sz[q];
-                        if (HILO) {
-                            dx += lx - slx[q];
-                            dy += ly - sly[q];
-                            dz += lz - slz[q];
-                        }
-                        pb_kernels<R>(dx, dy, dz, qx, qy, qz, snx[q], sny[q], snz[q], eps, inv_eps, kappa, K);
-                        s1 += K[0] * sdphi[q] + K[1] * sphi[q];
-                        s2 += K[2] * sdphi[q] + K[3] * sphi[q];
-                    }
-                }
-            }
-            acc1 += (double)s1;
-            acc2 += (double)s2;
-        }
-        if (act) {
-            double A = (double)ep[k].w;
-            ys[k] = 0.5 * (1.0 + eps_d) * A * xs[k] - A * acc1;
-            ys[nt + k] = 0.5 * (1.0 + 1.0 / eps_d) * A * xs[nt + k] - A * acc2;
-        }
+    __shared__ Near64Src sh[8];
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= ntiles) return;
+    Near64Src& S = sh[threadIdx.x >> 5];
+    int2 t = tiles[w];
+    int a0 = chunk_first[t.x], b0 = chunk_first[t.y];
+    int na = min(32, begin[chunk_leaf[t.x] + 1] - a0), nb = min(32, begin[chunk_leaf[t.y] + 1] - b0);
+    const bool diag = t.x == t.y;
+    const int side = nb > na;  // the lanes hold the second chunk
+    if (side) {
+        const int a = a0, n = na;
+        a0 = b0;
+        na = nb;
+        b0 = a;
+        nb = n;
     }
+    const double i4pi = 0.07957747154594767, inv_eps = 1.0 / eps;
+    if (lane < nb) {
+        const double4_32a p = ep[b0 + lane], n = en[b0 + lane];
+        S.x[lane] = p.x;
+        S.y[lane] = p.y;
+        S.z[lane] = p.z;
+        S.nx[lane] = n.x;
+        S.ny[lane] = n.y;
+        S.nz[lane] = n.z;
+        S.phi[lane] = p.w * xs[b0 + lane] * i4pi;  // 1 / (4 pi) rides on the densities
+        S.dphi[lane] = p.w * xs[nt + b0 + lane] * i4pi;
+    }
+    S.r1[lane] = S.r1[32 + lane] = 0.0;
+    S.r2[lane] = S.r2[32 + lane] = 0.0;
+    const bool act = lane < na;
+    const int k = a0 + (act ? lane : 0);
+    const double4_32a P = ep[k], Nn = en[k];
+    const double phi = act ? P.w * xs[k] * i4pi : 0.0, dphi = act ? P.w * xs[nt + k] * i4pi : 0.0;
+    __syncwarp();
+    double s1 = 0.0, s2 = 0.0;
+    const int g0 = lane / nb * nb;  // this lane's group of sums
+    int m = lane - g0;
+    for (int s = 0; s < nb; ++s) {
+        const bool same = diag && m == lane;  // the identical pair is the correction's
+        if (act && !same) {
+            const double dx = P.x - S.x[m], dy = P.y - S.y[m], dz = P.z - S.z[m];
+            const double ax = S.nx[m], ay = S.ny[m], az = S.nz[m];
+            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            const double ri = rsqrt(r2);
+            const double t1 = kappa * (r2 * ri);
+            const double e = exp(-t1);
+            const double e1 = fma(e, t1, e);                             // e^-t (1 + t)
+            const double c1n = e1 - 1.0;                                 // -c1
+            const double c3n = fma(e, fma(t1, t1 + 3.0, 3.0), -3.0);     // -c3
+            const double ri2 = ri * ri, ri3 = ri2 * ri;
+            const double nxd = fma(Nn.z, dz, fma(Nn.y, dy, Nn.x * dx));
+            const double nyd = fma(az, dz, fma(ay, dy, ax * dx));
+            const double nn = fma(Nn.z, az, fma(Nn.y, ay, Nn.x * ax));
+            const double f2 = ri3 * fma(eps, e1, -1.0), f3 = ri3 * fma(-inv_eps, e1, 1.0);
+            const double k1 = (1.0 - e) * ri;
+            const double k4 = ri3 * fma(c1n, nn, -c3n * (nxd * nyd * ri2));
+            const double sp = S.phi[m], sd = S.dphi[m];
+            s1 = fma(k1, sd, fma(nyd * f2, sp, s1));
+            s2 = fma(k4, sp, fma(-nxd * f3, sd, s2));
+            if (!diag) {
+                double* q1 = &S.r1[g0 + m];
+                double* q2 = &S.r2[g0 + m];
+                *q1 = fma(k1, dphi, fma(-nxd * f2, phi, *q1));
+                *q2 = fma(k4, phi, fma(nyd * f3, dphi, *q2));
+            }
+        }
+        __syncwarp();
+        if (++m == nb) m = 0;
+    }
+    double* out = part + (size_t)w * 128 + side * 64;
+    out[lane] = s1;
+    out[32 + lane] = s2;
+    if (!diag) {
+        out = part + (size_t)w * 128 + (side ^ 1) * 64;
+        double v1 = 0.0, v2 = 0.0;
+        if (lane < nb)
+            for (int g = lane; g - lane < 32; g += nb) {
+                v1 += S.r1[g];
+                v2 += S.r2[g];
+            }
+        out[lane] = v1;
+        out[32 + lane] = v2;
+    }
+}
+
+// One warp per chunk: y1 = 1/2 (1 + eps) A phi - A acc1, y2 = 1/2 (1 + 1/eps) A dphi - A acc2 with
+// acc the tiles' sums of the chunk (list[off[c]..off[c + 1]): 2 * tile + side) in list order.
+__global__ void __launch_bounds__(256) k_near64_sum(int nt, int nchunks, const int* __restrict__ off,
+                                                    const int* __restrict__ list, const int* __restrict__ chunk_leaf,
+                                                    const int* __restrict__ chunk_first, const int* __restrict__ begin,
+                                                    const double4_32a* __restrict__ ep, const double* __restrict__ part,
+                                                    const double* __restrict__ xs, double eps, double* __restrict__ ys)
+{
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (c >= nchunks) return;
+    const int k = chunk_first[c] + lane;
+    double a1 = 0.0, a2 = 0.0;
+#pragma unroll 4
+    for (int t = off[c]; t < off[c + 1]; ++t) {
+        const double* p = part + (size_t)list[t] * 64;
+        a1 += p[lane];
+        a2 += p[32 + lane];
+    }
+    if (k >= begin[chunk_leaf[c] + 1]) return;
+    const double A = ep[k].w;
+    ys[k] = 0.5 * (1.0 + eps) * A * xs[k] - A * a1;
+    ys[nt + k] = 0.5 * (1.0 + 1.0 / eps) * A * xs[nt + k] - A * a2;
+}
+
+// chunks, pair tiles, each chunk's list of tile sums, and the tiles' sums
+static int near64_setup(pb_ctx* c)
+{
+    const PbLevel& lv = c->lev[c->L];
+    const std::vector<int>&b = c->h_leaf_begin, &no = c->h_near_off, &ni = c->h_near_idx;
+    std::vector<int>&cl = c->h_up_i[0], &cf = c->h_up_i[1], &lst = c->h_up_i[4], &off = c->h_up_i[5];
+    std::vector<int2>& tl = c->h_up_i2;
+    cl.clear();
+    cf.clear();
+    tl.clear();
+    std::vector<int> first(lv.ncl + 1, 0);
+    for (int k = 0; k < lv.ncl; ++k) {
+        for (int s = b[k]; s < b[k + 1]; s += 32) {
+            cl.push_back(k);
+            cf.push_back(s);
+        }
+        first[k + 1] = (int)cl.size();
+    }
+    c->nchunks = (int)cl.size();
+    for (int k = 0; k < lv.ncl; ++k)
+        for (int a = first[k]; a < first[k + 1]; ++a)
+            for (int t = no[k]; t < no[k + 1]; ++t) {
+                const int c2 = ni[t];
+                if (c2 < k) continue;
+                for (int q = c2 == k ? a : first[c2]; q < first[c2 + 1]; ++q) tl.push_back(make_int2(a, q));
+            }
+    off.assign(c->nchunks + 1, 0);
+    for (const int2& t : tl) {
+        ++off[t.x + 1];
+        if (t.y != t.x) ++off[t.y + 1];
+    }
+    for (int k = 0; k < c->nchunks; ++k) off[k + 1] += off[k];
+    lst.resize(off[c->nchunks]);
+    std::vector<int> at(off.begin(), off.end() - 1);
+    for (size_t t = 0; t < tl.size(); ++t) {
+        lst[at[tl[t].x]++] = (int)(2 * t);
+        if (tl[t].y != tl[t].x) lst[at[tl[t].y]++] = (int)(2 * t + 1);
+    }
+    if (tl.size() > 0x3fffffff) return pb_fail(c, PB_ERR_NOMEM, "near setup: too many pair tiles");
+    c->near_nitems = (int)tl.size();
+    c->chunk_leaf = (int*)pb_alloc(c, sizeof(int) * cl.size());
+    c->chunk_first = (int*)pb_alloc(c, sizeof(int) * cf.size());
+    c->near_tiles2 = (int2*)pb_alloc(c, sizeof(int2) * tl.size());
+    c->near_off = (int*)pb_alloc(c, sizeof(int) * off.size());
+    c->near_list = (int*)pb_alloc(c, sizeof(int) * lst.size());
+    c->near_part = (double*)pb_alloc(c, sizeof(double) * 128 * tl.size());
+    if (!c->chunk_leaf || !c->chunk_first || !c->near_tiles2 || !c->near_off || !c->near_list || !c->near_part)
+        return pb_fail(c, PB_ERR_NOMEM, "near setup: out of memory");
+    auto up = [&](void* d, const void* h, size_t n) { return cudaMemcpyAsync(d, h, n, cudaMemcpyHostToDevice, c->st); };
+    PB_CUDA(c, up(c->chunk_leaf, cl.data(), sizeof(int) * cl.size()));
+    PB_CUDA(c, up(c->chunk_first, cf.data(), sizeof(int) * cf.size()));
+    PB_CUDA(c, up(c->near_tiles2, tl.data(), sizeof(int2) * tl.size()));
+    PB_CUDA(c, up(c->near_off, off.data(), sizeof(int) * off.size()));
+    PB_CUDA(c, up(c->near_list, lst.data(), sizeof(int) * lst.size()));
+    return PB_OK;
 }
 
 // ---------- mixed precision near field ----------
@@ -521,7 +624,8 @@ __global__ void k_corrections(int nt, const int* __restrict__ toff, const int* _
 // chunks of at most 32 targets per leaf and the packed source buffers (mixed precision)
 int pb_near_setup(pb_ctx* c)
 {
-    if (c->prm.precision != PB_MIXED) return PB_OK;
+    // (with a regular rule of order > 1 the FP64 near field runs on its points, pb_near_q_apply)
+    if (c->prm.precision != PB_MIXED) return c->q2 > 1 ? PB_OK : near64_setup(c);
     const PbLevel& lv = c->lev[c->L];
     const std::vector<int>& b = c->h_leaf_begin;  // the leaf ranges, read back by the tree build
     std::vector<int>& cl = c->h_up_i[0];
@@ -596,10 +700,15 @@ int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
             c->near_sn, c->e32l, eps, c->prm.kappa, ys);
         PB_LAUNCH(c);
         k_near_finish<<<(nt + 255) / 256, 256, 0, c->st>>>(nt, c->e64p, xs, eps, ys);
-    } else
-        k_near<double, double4_32a, false><<<lv.ncl, NEAR_T, 0, c->st>>>(c->nt, lv.begin, lv.near_off,
-                                                                         lv.near_idx, c->e64p, c->e64n, nullptr, xs,
-                                                                         eps, c->prm.kappa, ys);
+    } else {
+        k_near64<<<(unsigned)(((long long)c->near_nitems * 32 + 255) / 256), 256, 0, c->st>>>(
+            c->nt, c->near_nitems, c->near_tiles2, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p, c->e64n, xs, eps,
+            c->prm.kappa, c->near_part);
+        PB_LAUNCH(c);
+        k_near64_sum<<<(unsigned)(((long long)c->nchunks * 32 + 255) / 256), 256, 0, c->st>>>(
+            c->nt, c->nchunks, c->near_off, c->near_list, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p,
+            c->near_part, xs, eps, ys);
+    }
     PB_LAUNCH(c);
     return PB_OK;
 }

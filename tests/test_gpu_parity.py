@@ -312,3 +312,27 @@ def test_tiny_and_ragged_meshes():
             assert _rel(y.cpu().numpy(), yo) < 1e-10
         finally:
             pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("leaf,levels", [(1000, 1), (1, 3), (3, 2), (40, 0), (70, 0)])
+@pytest.mark.parametrize("part", [0, 1])
+def test_fp64_pair_tiles_ragged_leaves(leaf, levels, part):
+    # chunks of 1 to 32 elements: leaves of one and a few elements, remainders on both sides of a
+    # tile, one leaf of many chunks; bar as above (FP64 mode within 1e-10 of the oracle FMM)
+    V, T = inputs.perturbed_sphere(3, 2.0, 0.2, seed=17)
+    T = T[:1277] if levels == 0 else T
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    ctx = _ctx(m, eta0=0.8, leaf_size=leaf, levels=levels, p=6, precision=pb.PB_FP64, precond=pb.PB_PRECOND_DIAG)
+    try:
+        tr = fmm.Tree(V, T, leaf_size=leaf, eta0=0.8, levels=levels) if levels else fmm.Tree(V, T, leaf_size=leaf, eta0=0.8)
+        x = inputs.random_density(m.nt, leaf)
+        y = torch.empty(2 * m.nt, device="cuda", dtype=torch.float64)
+        pb.pb_matvec_part(ctx, _dev(x), y, part)
+        if part == 0:
+            ph = dense.Phys(1.0, 80.0, KAP, qs=3)
+            assert _rel(y.cpu().numpy(), fmm.matvec(tr, V, T, x, ph, 6)) < 1e-10
+        z = torch.empty_like(y)
+        pb.pb_matvec_part(ctx, _dev(x), z, part)
+        assert torch.equal(y, z)  # no atomics: the same product twice is the same bits
+    finally:
+        pb.pb_destroy(ctx)
