@@ -3,12 +3,12 @@
 For a fixed order P the MtL sum of eqcoeff, written as
     a! lam^a = sum_{|a| + |b| <= P} D^{a+b} G(d) * M^b,   M^b = (-1)^|b| m^b / b!,
 has a fixed set of (gamma = a + b, a, b) triples. Emitting them as explicit statements lets
-the compiler keep the local coefficients in registers. Each body handles the multi-indices
-a in one range [a0, a1) (the coefficients can be split into passes of at most SPLIT so
-that one pass fits in registers), walks gamma in layout order, loads D^gamma from the
-interleaved slot layout (Dl[gamma * 32]) in groups of GROUP so that several loads are in
-flight before their values are used, and reads the scaled moments from shared memory
-(Ms[b * 32], the interleaved chunk layout).
+the compiler keep the local coefficients in registers. M2LBody<P, W> (FP64 kernel) handles one of
+NBODY[P] sets of multi-indices a with equal FMA counts (at most 42 coefficients, so that a set's
+accumulators fit in registers), walks gamma in layout order, loads D^gamma from the interleaved
+slot layout (Dl[gamma * 32]) in groups of GROUP so that several loads are in flight before their
+values are used, and reads the scaled moments from shared memory (Ms[b * 33]) for every FMA
+(volatile: kept in registers across FMAs they spilled the accumulators).
 
 M2LWarp<P, W> is the register-blocked two-warp variant used by the FP32 kernel: warp W
 accumulates half of the local coefficients (equal FMA counts), the moments of a block of
@@ -23,7 +23,7 @@ Run: python gen_m2l.py > m2l_unrolled.cuh  (the output is committed beside this 
 from math import comb
 
 ORDERS = (4, 6, 8)
-SPLIT = 165
+NBODY = {4: 1, 6: 2, 8: 4}
 GROUP = 4
 # two-warp register-blocked bodies (FP32 kernel): the local coefficients are split between two
 # warps with equal FMA counts, and each warp holds the moments of MBLOCK multi-indices at a
@@ -44,21 +44,17 @@ def multi_indices(p):
     return out
 
 
-def passes(T):
-    return [(a0, min(T, a0 + SPLIT)) for a0 in range(0, T, SPLIT)]
-
-
-def body(P, a0, a1):
+def body(P, aset):
     idx = multi_indices(P)
     pos = {t: i for i, t in enumerate(idx)}
-    work = []  # (gamma, [(alpha - a0, beta)])
+    work = []  # (gamma, [(k, beta)])
     for g, gm in enumerate(idx):
         splits = []
-        for ia in range(a0, a1):
+        for k, ia in enumerate(aset):
             al = idx[ia]
             be = (gm[0] - al[0], gm[1] - al[1], gm[2] - al[2])
             if min(be) >= 0:
-                splits.append((ia - a0, pos[be]))
+                splits.append((k, pos[be]))
         if splits:
             work.append((g, splits))
     out = []
@@ -68,18 +64,18 @@ def body(P, a0, a1):
             out.append(f"        d{k} = Dl[{g * 32}];")
         for k, (_, splits) in enumerate(grp):
             for ia, ib in splits:
-                out.append(f"        L[{ia}] += d{k} * Ms[{ib * 32}];")
+                out.append(f"        L[{ia}] += d{k} * Ms[{ib * MSTRIDE}];")
     return out
 
 
-def warp_sets(P):
-    """Split the multi-indices a between NWARP warps so that each gets the same number of
+def warp_sets(P, nwarp=NWARP):
+    """Split the multi-indices a between nwarp warps so that each gets the same number of
     (a, b) pairs: a pairs with C(P - |a| + 3, 3) moments, so low orders are heavy. Greedy,
     heaviest first, ties to the lower warp; each set in layout order."""
     idx = multi_indices(P)
     wt = [comb(P - sum(a) + 3, 3) for a in idx]
-    load = [0] * NWARP
-    sets = [[] for _ in range(NWARP)]
+    load = [0] * nwarp
+    sets = [[] for _ in range(nwarp)]
     for i in sorted(range(len(idx)), key=lambda i: (-wt[i], i)):
         k = load.index(min(load))
         load[k] += wt[i]
@@ -128,29 +124,33 @@ def main():
         "// Generated by gen_m2l.py -- straight-line MtL contraction bodies. Do not edit.",
         "#pragma once",
         "",
-        f"#define M2L_SPLIT {SPLIT}",
-        "",
-        "template <int P, int PASS>",
-        "struct M2LBody;",
-        "",
+        "// FP64 bodies: the sets of local coefficients (warps) and the largest set",
         "template <int P>",
-        "struct M2LPassCount;",
+        "struct M2LBodies;",
+        "template <int P, int W>",
+        "struct M2LBody;",
         "",
     ]
     for P in ORDERS:
-        T = len(multi_indices(P))
-        ps = passes(T)
-        lines.append(f"template <>\nstruct M2LPassCount<{P}> {{\n    static constexpr int n = {len(ps)};\n}};\n")
-        for k, (a0, a1) in enumerate(ps):
+        sets = warp_sets(P, NBODY[P])
+        lines.append(f"template <>\nstruct M2LBodies<{P}> {{\n    static constexpr int n = {NBODY[P]}, "
+                     f"most = {max(map(len, sets))};\n}};\n")
+        for w, aset in enumerate(sets):
             lines += [
                 "template <>",
-                f"struct M2LBody<{P}, {k}> {{",
+                f"struct M2LBody<{P}, {w}> {{",
+                f"    static constexpr int n = {len(aset)};",
+                "    static __device__ __forceinline__ int alpha(int k)",
+                "    {",
+                f"        constexpr short a[{len(aset)}] = {{{', '.join(str(x) for x in aset)}}};",
+                "        return a[k];",
+                "    }",
                 "    template <class R>",
-                "    static __device__ __forceinline__ void run(const R* __restrict__ Dl, const R* __restrict__ Ms, R* L)",
+                "    static __device__ __forceinline__ void run(const R* __restrict__ Dl, const volatile R* Ms, R* L)",
                 "    {",
                 "        R " + ", ".join(f"d{i}" for i in range(GROUP)) + ";",
             ]
-            lines += body(P, a0, a1)
+            lines += body(P, aset)
             lines += ["    }", "};", ""]
     lines += ["template <int P, int W>", "struct M2LWarp;", ""]
     for P in ORDERS:

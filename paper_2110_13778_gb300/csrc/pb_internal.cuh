@@ -51,8 +51,6 @@ struct PbLevel {
     long long nslots = 0;
     void* D0 = nullptr;      // derivatives of G0, working precision
     void* Dk = nullptr;      // derivatives of Gk
-    void* Mg0 = nullptr;     // scaled source moments gathered into the slot layout (per product)
-    void* Mgk = nullptr;
     void* Mp0 = nullptr;     // mixed MtL: the sums of the runs that cross a chunk edge, [nr][chunk][2][T]
     void* Mpk = nullptr;
     int* slot_tgt = nullptr; // [nslots] target cluster of each slot (table setup)
