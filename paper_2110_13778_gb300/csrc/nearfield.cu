@@ -26,7 +26,7 @@
 #include "pb_internal.cuh"
 
 
-#define NEAR_ITEM 6    // pair tiles per warp of the mixed-precision near field
+#define NEAR_ITEM 6    // most pair tiles per warp of the mixed-precision near field
 #define NEAR_ITEM_M 8  // directed tiles per warp of the several-vector near field
 
 // ---------- FP64 near field ----------
@@ -190,6 +190,7 @@ static int near64_setup(pb_ctx* c)
                 if (c2 < k) continue;
                 for (int q = c2 == k ? a : first[c2]; q < first[c2 + 1]; ++q) tl.push_back(make_int2(a, q));
             }
+    if (tl.size() > 0x3fffffff) return pb_fail(c, PB_ERR_NOMEM, "near setup: too many pair tiles");
     off.assign(c->nchunks + 1, 0);
     for (const int2& t : tl) {
         ++off[t.x + 1];
@@ -202,7 +203,6 @@ static int near64_setup(pb_ctx* c)
         lst[at[tl[t].x]++] = (int)(2 * t);
         if (tl[t].y != tl[t].x) lst[at[tl[t].y]++] = (int)(2 * t + 1);
     }
-    if (tl.size() > 0x3fffffff) return pb_fail(c, PB_ERR_NOMEM, "near setup: too many pair tiles");
     c->near_nitems = (int)tl.size();
     c->chunk_leaf = (int*)pb_alloc(c, sizeof(int) * cl.size());
     c->chunk_first = (int*)pb_alloc(c, sizeof(int) * cf.size());
@@ -248,8 +248,8 @@ __global__ void k_near_pack(int nt, const float4* __restrict__ e32p, const float
 // l pairs A_l with B_((l + s) mod nb) and B_((l + s + h) mod nb), h = ceil(nb / 2), and keeps
 // the forward terms. The reverse terms of a full tile of another chunk (nb = 32) ride in
 // registers that move one lane down after every step (shuffles), so that after 16 steps lane l
-// holds the sums of sources (l + 16) mod 32 and l; partial tiles add them to B's shared-memory
-// accumulators instead (FP32 shared atomics). Forward sums of a chunk and reverse sums of a
+// holds the sums of sources (l + 16) mod 32 and l; in partial tiles lane j gathers those of source
+// j by shuffles. Forward sums of a chunk and reverse sums of a
 // tile are FP32, added into FP64 (atomics for the reverse terms and the final forward sums; ys
 // starts at zero). The tile of A with itself keeps only the forward terms and drops the
 // identical pair.
@@ -259,22 +259,48 @@ __global__ void k_near_pack(int nt, const float4* __restrict__ e32p, const float
 //
 // Packed pairs: entry m of a staged tile holds source m in the low halves and source
 // (m + h) mod nb in the high halves, as F0 = (x, y), F1 = (z, A phi), F2 = (n_x, n_y),
-// F3 = (n_z, -A dphi) of the high coordinate parts and F4 = (x, y), F5 = (z, 0) of the low
+// F3 = (n_z, -A dphi) of the high coordinate parts and F4 = (x, y), F5 = (z) of the low
 // parts. Every FP32 operation of the two pairs of a step is one f32x2 instruction; only the
 // reciprocal square root, the exponential and the branch of the screening function run per
 // half. (The packed instructions do not raise the FP32 rate; they halve the issue slots that
 // bound this loop.)
+//
+// Bound: the FMA pipe (two cycles per packed instruction; 62 of them per step of 64 pairs, 69 %
+// busy on 737,280 elements of 170 per leaf). Against shared-memory sums and the general screening
+// function in every tile: 3090 -> 2567 us there, 202 -> 158 us on 81,920 elements (leaves of 71:
+// 20 % of the steps are remainder tiles), 35 -> 12 us on 1280. Blocks of four warps, because items
+// differ in length; seven per SM (72 registers) is the best of 5 to 8 by 1 to 4 %.
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 struct NearTgt2 {
     f2x px, py, pz, lx, ly, lz, nx, ny, nz, phi, dphi;
 };
 
 // s1, s2 += forward terms; q1n -= first reverse term, q2 += second reverse term (per half).
-// bump is added to r^2 of dropped pairs (so that r stays finite), scale = 1 / (4 pi) or 0.
-template <bool BUMP>
-__device__ __forceinline__ void near_pair_x2(const NearTgt2& T, const float4* __restrict__ e, f2x bump, f2x scale,
-                                             f2x eps2, f2x nieps2, f2x kappa2, f2x& s1, f2x& s2, f2x& q1n, f2x& q2)
+// BUMP: bump is added to r^2 of dropped pairs (so that r stays finite); scale = 1 / (4 pi) or 0.
+// The Taylor series of the screening function (nine of 64 packed operations and the selections) is
+// needed where kappa r < 0.125 only: FAR says that no pair of the tile is that close; other tiles ask
+// the warp at every step. The bare (flushing) reciprocal square root and exponential give the bits of
+// rsqrtf and __expf wherever those matter: r^2 is no subnormal number for distinct centres, and
+// e^-t - 1 is -1 for a flushed e^-t as for a subnormal one.
+template <bool BUMP, bool FAR>
+__device__ __forceinline__ void near_pair_x2(const NearTgt2& T, const float4* __restrict__ e,
+                                             const float2* __restrict__ e5, f2x bump, f2x scale, f2x eps2, f2x nieps2,
+                                             f2x kappa2, f2x& s1, f2x& s2, f2x& q1n, f2x& q2)
 {
-    const float4 g0 = e[0], g1 = e[32], g2 = e[64], g3 = e[96], g4 = e[128], g5 = e[160];
+    const float4 g0 = e[0], g1 = e[32], g2 = e[64], g3 = e[96], g4 = e[128];
+    const float2 g5 = *e5;
     const f2x ax = x2_pack(g0.x, g0.y), ay = x2_pack(g0.z, g0.w), az = x2_pack(g1.x, g1.y);
     const f2x aphi = x2_pack(g1.z, g1.w);
     const f2x bx = x2_pack(g2.x, g2.y), by = x2_pack(g2.z, g2.w), bz = x2_pack(g3.x, g3.y);
@@ -288,28 +314,35 @@ __device__ __forceinline__ void near_pair_x2(const NearTgt2& T, const float4* __
     if (BUMP) r2 = x2_add(r2, bump);
     float ra, rb;
     x2_unpack(r2, ra, rb);
-    const f2x rinv = x2_pack(rsqrtf(ra), rsqrtf(rb));
+    const f2x rinv = x2_pack(rsqrt_ftz(ra), rsqrt_ftz(rb));
     const f2x tt = x2_mul(kappa2, x2_mul(r2, rinv));
-    // g / t^2 = 1/2 - t/6 + t^2/24 - ... (the Taylor series of e^-t - 1 + t), for small t
-    f2x sg = x2_fma(x2_dup(1.f / 40320.f), tt, x2_dup(-1.f / 5040.f));
-    sg = x2_fma(sg, tt, x2_dup(1.f / 720.f));
-    sg = x2_fma(sg, tt, x2_dup(-1.f / 120.f));
-    sg = x2_fma(sg, tt, x2_dup(1.f / 24.f));
-    sg = x2_fma(sg, tt, x2_dup(-1.f / 6.f));
-    sg = x2_fma(sg, tt, x2_dup(0.5f));
-    const f2x gs = x2_mul(x2_mul(sg, tt), tt);
-    float ta, tb;
-    x2_unpack(tt, ta, tb);
-    const f2x ed = x2_add(x2_pack(__expf(-ta), __expf(-tb)), mone);
-    const f2x ga = x2_add(ed, tt), eb = x2_sub(gs, tt);
-    float gsa, gsb, gaa, gab, eba, ebb, eda, edb;
-    x2_unpack(gs, gsa, gsb);
-    x2_unpack(ga, gaa, gab);
-    x2_unpack(eb, eba, ebb);
-    x2_unpack(ed, eda, edb);
-    const bool sa = ta < 0.125f, sb = tb < 0.125f;
-    const f2x g = x2_pack(sa ? gsa : gaa, sb ? gsb : gab);
-    const f2x E = x2_pack(sa ? eba : eda, sb ? ebb : edb);
+    float xa, xb;
+    x2_unpack(x2_mul(tt, x2_dup(-1.4426950408889634f)), xa, xb);
+    f2x E = x2_add(x2_pack(ex2_ftz(xa), ex2_ftz(xb)), mone);
+    f2x g = x2_add(E, tt);
+    if (!FAR) {
+        float ta, tb;
+        x2_unpack(tt, ta, tb);
+        const bool sa = ta < 0.125f, sb = tb < 0.125f;
+        if (__any_sync(0xffffffffu, sa || sb)) {
+            // g / t^2 = 1/2 - t/6 + t^2/24 - ... (the Taylor series of e^-t - 1 + t), for small t
+            f2x sg = x2_fma(x2_dup(1.f / 40320.f), tt, x2_dup(-1.f / 5040.f));
+            sg = x2_fma(sg, tt, x2_dup(1.f / 720.f));
+            sg = x2_fma(sg, tt, x2_dup(-1.f / 120.f));
+            sg = x2_fma(sg, tt, x2_dup(1.f / 24.f));
+            sg = x2_fma(sg, tt, x2_dup(-1.f / 6.f));
+            sg = x2_fma(sg, tt, x2_dup(0.5f));
+            const f2x gs = x2_mul(x2_mul(sg, tt), tt);
+            const f2x eb = x2_sub(gs, tt);
+            float gsa, gsb, gaa, gab, eba, ebb, eda, edb;
+            x2_unpack(gs, gsa, gsb);
+            x2_unpack(g, gaa, gab);
+            x2_unpack(eb, eba, ebb);
+            x2_unpack(E, eda, edb);
+            g = x2_pack(sa ? gsa : gaa, sb ? gsb : gab);
+            E = x2_pack(sa ? eba : eda, sb ? ebb : edb);
+        }
+    }
     const f2x tE = x2_mul(tt, E);
     const f2x c1n = x2_add(g, tE);                                            // -c1
     const f2x c3n = x2_fma(tE, x2_add(three, tt), x2_fma(tt, tt, x2_mul(three, g)));  // -c3
@@ -339,16 +372,84 @@ __device__ __forceinline__ f2x x2_shfl_down1(f2x v, int lane)
     return x2_pack(a, b);
 }
 
+// a full tile of another chunk: lane l meets sources (l + s) mod 32 and (l + s + 16) mod 32 at step
+// s; the reverse sums move one lane down after every step. t1, t2: the sums of source `lane`.
+template <bool FAR>
+__device__ __forceinline__ void near_tile_full(const NearTgt2& T, const float4* F, const float2* F5, int lane, f2x sc,
+                                               f2x eps2, f2x nieps2, f2x kappa2, f2x& s1, f2x& s2, float& t1, float& t2)
+{
+    f2x q1n = x2_dup(0.f), q2 = q1n;
+    int m = lane;
+#pragma unroll 4
+    for (int s = 0; s < 16; ++s) {
+        near_pair_x2<false, FAR>(T, F + m, F5 + m, q1n, sc, eps2, nieps2, kappa2, s1, s2, q1n, q2);
+        q1n = x2_shfl_down1(q1n, lane);
+        q2 = x2_shfl_down1(q2, lane);
+        m = (m + 1) & 31;
+    }
+    // lane l: the low halves belong to source (l + 16) mod 32, the high halves to l
+    float a1, b1, a2, b2;
+    x2_unpack(q1n, a1, b1);
+    x2_unpack(q2, a2, b2);
+    t1 = -(b1 + __shfl_sync(0xffffffffu, a1, (lane + 16) & 31));
+    t2 = b2 + __shfl_sync(0xffffffffu, a2, (lane + 16) & 31);
+}
+
+// a tile with fewer than 32 sources: lane j < nb gathers the reverse terms of source j by shuffles,
+// in the order (step, low half before high half, lane), one FP32 sum per source. (Shared-memory
+// atomics, four per step and lane, did this before; FP32 ones are compare-and-swap loops.)
+template <bool FAR>
+__device__ __forceinline__ void near_tile_part(const NearTgt2& T, const float4* F, const float2* F5, int lane, int nb,
+                                               int na, bool act, f2x eps2, f2x nieps2, f2x kappa2, f2x& s1, f2x& s2,
+                                               float& t1, float& t2)
+{
+    const float i4pi = 0.07957747154594767f;
+    const int h = (nb + 1) >> 1;
+    const f2x zero = x2_dup(0.f), sc = x2_dup(act ? i4pi : 0.f), scl = x2_pack(act ? i4pi : 0.f, 0.f);
+    int m = lane % nb;
+    // the lane that meets source `lane` in the low half at step s, and in the high half
+    int p = m, ph = m - h < 0 ? m - h + nb : m - h;
+    t1 = t2 = 0.f;
+    for (int s = 0; s < h; ++s) {
+        f2x q1n = zero, q2 = zero;
+        // for odd nb the high half of the last step repeats a source: dropped
+        near_pair_x2<false, FAR>(T, F + m, F5 + m, zero, (nb & 1) && s == h - 1 ? scl : sc, eps2, nieps2, kappa2, s1, s2,
+                                 q1n, q2);
+        float a1, b1, a2, b2;
+        x2_unpack(q1n, a1, b1);
+        x2_unpack(q2, a2, b2);
+        for (int g = 0; g < na; g += nb) {
+            const float v1 = __shfl_sync(0xffffffffu, a1, (p + g) & 31), v2 = __shfl_sync(0xffffffffu, a2, (p + g) & 31);
+            if (p + g < 32) {
+                t1 -= v1;
+                t2 += v2;
+            }
+        }
+        for (int g = 0; g < na; g += nb) {
+            const float v1 = __shfl_sync(0xffffffffu, b1, (ph + g) & 31), v2 = __shfl_sync(0xffffffffu, b2, (ph + g) & 31);
+            if (ph + g < 32) {
+                t1 -= v1;
+                t2 += v2;
+            }
+        }
+        m = m + 1 == nb ? 0 : m + 1;
+        p = p == 0 ? nb - 1 : p - 1;
+        ph = ph == 0 ? nb - 1 : ph - 1;
+    }
+}
+
+#define NEAR_FAR (1 << 30)  // flag of a tile (k_near_flag): kappa r >= 0.125 for all its pairs
+#define NEAR_W 4            // warps per block
 template <int Q2>
-__global__ void __launch_bounds__(256, 3) k_near_tile(int nt, int nitems, const int4* __restrict__ items,
+__global__ void __launch_bounds__(32 * NEAR_W, 7) k_near_tile(int nt, int nitems, const int4* __restrict__ items,
                                                     const int* __restrict__ tiles, const int* __restrict__ chunk_leaf,
                                                     const int* __restrict__ chunk_first, const int* __restrict__ begin,
                                                     const float4* __restrict__ sp, const float4* __restrict__ sn,
                                                     const float4* __restrict__ sl, double eps_d, double kappa_d,
                                                     double* __restrict__ ys)
 {
-    __shared__ float4 fq[8][6 * 32];
-    __shared__ float rv1[8][32], rv2[8][32];
+    __shared__ float4 fq[NEAR_W][5 * 32];
+    __shared__ float2 fq5[NEAR_W][32];
     const float i4pi = 0.07957747154594767f;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
@@ -356,8 +457,9 @@ __global__ void __launch_bounds__(256, 3) k_near_tile(int nt, int nitems, const 
     const int4 item = items[w];
     const int ca = item.x;
     const int c = chunk_leaf[ca], a0 = chunk_first[ca];
+    const int na = min(32, begin[c + 1] - a0);
     const int k = a0 + lane;
-    const bool act = k < begin[c + 1];
+    const bool act = lane < na;
     const int kk = act ? k : a0;
     NearTgt2 T;
     {
@@ -378,10 +480,10 @@ __global__ void __launch_bounds__(256, 3) k_near_tile(int nt, int nitems, const 
     const f2x zero = x2_dup(0.f);
     double acc1 = 0.0, acc2 = 0.0;
     float4* F = fq[wi];
+    float2* F5 = fq5[wi];
     for (int ti = item.y; ti < item.z; ++ti) {
-        const int cb = tiles[ti];
+        const int tv = tiles[ti], cb = tv & (NEAR_FAR - 1);
         const int b0 = chunk_first[cb], se = begin[chunk_leaf[cb] + 1];
-        const bool diag = cb == ca;
         const int nb = min(32, se - b0);
         if (nb <= 0) continue;  // no chunk is empty; the test keeps the indexing below in range
         const int h = (nb + 1) >> 1;
@@ -405,65 +507,41 @@ __global__ void __launch_bounds__(256, 3) k_near_tile(int nt, int nitems, const 
                 F[64 + lane] = make_float4(n.x, Nx, n.y, Ny);
                 F[96 + lane] = make_float4(n.z, Nz, -n.w, -Nw);
                 F[128 + lane] = make_float4(lo.x, Lx, lo.y, Ly);
-                F[160 + lane] = make_float4(lo.z, Lz, 0.f, 0.f);
+                F5[lane] = make_float2(lo.z, Lz);
             }
             __syncwarp();
         }
         f2x s1 = zero, s2 = zero;
-        if (!diag && nb == 32) {
-            // full tile of another chunk: lane l meets sources (l + s) mod 32 and (l + s + 16)
-            // mod 32 at step s; the reverse sums move one lane down after every step
-            const f2x sc = x2_dup(act ? i4pi : 0.f);
-            f2x q1n = zero, q2 = zero;
-            int m = lane;
-#pragma unroll 4
-            for (int s = 0; s < 16; ++s) {
-                near_pair_x2<false>(T, F + m, zero, sc, eps2, nieps2, kappa2, s1, s2, q1n, q2);
-                q1n = x2_shfl_down1(q1n, lane);
-                q2 = x2_shfl_down1(q2, lane);
-                m = (m + 1) & 31;
-            }
-            // lane l: the low halves belong to source (l + 16) mod 32, the high halves to l
-            float a1, b1, a2, b2;
-            x2_unpack(q1n, a1, b1);
-            x2_unpack(q2, a2, b2);
-            const float t1 = b1 + __shfl_sync(0xffffffffu, a1, (lane + 16) & 31);
-            const float t2 = b2 + __shfl_sync(0xffffffffu, a2, (lane + 16) & 31);
-            atomicAdd(&ys[b0 + lane], -(double)t1);
-            atomicAdd(&ys[nt + b0 + lane], (double)t2);
-        } else {
-            rv1[wi][lane] = 0.f;
-            rv2[wi][lane] = 0.f;
-            __syncwarp();
+        if (cb == ca) {
+            // the chunk with itself: forward terms only, without the identical pair (the
+            // correction's) or the pairs of one element's points
             int m = lane % nb;
             int m2 = m + h;
             if (m2 >= nb) m2 -= nb;
             const bool odd = nb & 1;
             for (int s = 0; s < h; ++s) {
-                // drop the identical pair (the correction's), padding targets and, for odd nb,
-                // the repeated source of the last step
-                const bool okl = act && !(diag && (Q2 == 1 ? m == lane : m / Q2 == lane / Q2));
-                const bool okh = act && !(odd && s == h - 1) && !(diag && (Q2 == 1 ? m2 == lane : m2 / Q2 == lane / Q2));
-                const f2x bump = x2_pack(okl ? 0.f : 1.f, okh ? 0.f : 1.f);
-                const f2x sc = x2_pack(okl ? i4pi : 0.f, okh ? i4pi : 0.f);
+                const bool okl = act && !(Q2 == 1 ? m == lane : m / Q2 == lane / Q2);
+                const bool okh = act && !(odd && s == h - 1) && !(Q2 == 1 ? m2 == lane : m2 / Q2 == lane / Q2);
                 f2x q1n = zero, q2 = zero;
-                near_pair_x2<true>(T, F + m, bump, sc, eps2, nieps2, kappa2, s1, s2, q1n, q2);
-                if (!diag) {
-                    float a1, b1, a2, b2;
-                    x2_unpack(q1n, a1, b1);
-                    x2_unpack(q2, a2, b2);
-                    atomicAdd(&rv1[wi][m], -a1);
-                    atomicAdd(&rv1[wi][m2], -b1);
-                    atomicAdd(&rv2[wi][m], a2);
-                    atomicAdd(&rv2[wi][m2], b2);
-                }
+                near_pair_x2<true, false>(T, F + m, F5 + m, x2_pack(okl ? 0.f : 1.f, okh ? 0.f : 1.f),
+                                          x2_pack(okl ? i4pi : 0.f, okh ? i4pi : 0.f), eps2, nieps2, kappa2, s1, s2, q1n,
+                                          q2);
                 m = m + 1 == nb ? 0 : m + 1;
                 m2 = m2 + 1 == nb ? 0 : m2 + 1;
             }
-            __syncwarp();
-            if (!diag && lane < nb) {
-                atomicAdd(&ys[b0 + lane], (double)rv1[wi][lane]);
-                atomicAdd(&ys[nt + b0 + lane], (double)rv2[wi][lane]);
+        } else {
+            float t1, t2;
+            if (nb == 32) {
+                const f2x sc = x2_dup(act ? i4pi : 0.f);
+                if (tv & NEAR_FAR) near_tile_full<true>(T, F, F5, lane, sc, eps2, nieps2, kappa2, s1, s2, t1, t2);
+                else near_tile_full<false>(T, F, F5, lane, sc, eps2, nieps2, kappa2, s1, s2, t1, t2);
+            } else {
+                if (tv & NEAR_FAR) near_tile_part<true>(T, F, F5, lane, nb, na, act, eps2, nieps2, kappa2, s1, s2, t1, t2);
+                else near_tile_part<false>(T, F, F5, lane, nb, na, act, eps2, nieps2, kappa2, s1, s2, t1, t2);
+            }
+            if (lane < nb) {
+                atomicAdd(&ys[b0 + lane], (double)t1);
+                atomicAdd(&ys[nt + b0 + lane], (double)t2);
             }
         }
         float a, b;
@@ -476,6 +554,59 @@ __global__ void __launch_bounds__(256, 3) k_near_tile(int nt, int nitems, const 
         atomicAdd(&ys[k], acc1);
         atomicAdd(&ys[nt + k], acc2);
     }
+}
+
+// Build: bounding box of every chunk's centres (or points), one warp per chunk
+__global__ void k_chunk_box(int nchunks, const int* __restrict__ chunk_leaf, const int* __restrict__ chunk_first,
+                            const int* __restrict__ begin, const double4_32a* __restrict__ ep, double* __restrict__ box)
+{
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (c >= nchunks) return;
+    const int k = min(chunk_first[c] + lane, begin[chunk_leaf[c] + 1] - 1);
+    const double4_32a p = ep[k];
+    double lo[3] = {p.x, p.y, p.z}, hi[3] = {p.x, p.y, p.z};
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[a] = fmin(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+            hi[a] = fmax(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+        }
+    if (lane < 3) box[6 * (size_t)c + lane] = lane == 0 ? lo[0] : lane == 1 ? lo[1] : lo[2];
+    else if (lane < 6) box[6 * (size_t)c + lane] = lane == 3 ? hi[0] : lane == 4 ? hi[1] : hi[2];
+}
+
+// Build: NEAR_FAR on the tiles whose chunks' boxes are at least 0.125 / kappa apart, with a margin
+// of 1e-5 for the FP32 rounding of kappa r in the kernel; one thread per work item
+__global__ void k_near_flag(int nitems, const int4* __restrict__ items, const double* __restrict__ box, double kappa,
+                            int* __restrict__ tiles)
+{
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= nitems) return;
+    const int4 item = items[w];
+    const double* A = box + 6 * (size_t)item.x;
+    for (int t = item.y; t < item.z; ++t) {
+        const int cb = tiles[t] & (NEAR_FAR - 1);
+        const double* B = box + 6 * (size_t)cb;
+        double d2 = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            const double d = fmax(0.0, fmax(A[a] - B[3 + a], B[a] - A[3 + a]));
+            d2 += d * d;
+        }
+        tiles[t] = cb | (kappa * sqrt(d2) >= 0.125 * (1.0 + 1e-5) ? NEAR_FAR : 0);
+    }
+}
+
+static int near_flags(pb_ctx* c, int nchunks, const int* chunk_leaf, const int* chunk_first, const int* begin,
+                      const double4_32a* ep, int nitems, const int4* items, int* tiles)
+{
+    double* box = (double*)pb_alloc(c, sizeof(double) * 6 * (size_t)nchunks);
+    if (!box) return pb_fail(c, PB_ERR_NOMEM, "near setup: out of memory");
+    k_chunk_box<<<(unsigned)(((long long)nchunks * 32 + 255) / 256), 256, 0, c->st>>>(nchunks, chunk_leaf, chunk_first,
+                                                                                        begin, ep, box);
+    PB_LAUNCH(c);
+    k_near_flag<<<(nitems + 127) / 128, 128, 0, c->st>>>(nitems, items, box, c->prm.kappa, tiles);
+    PB_LAUNCH(c);
+    return PB_OK;
 }
 
 // ---------- several right-hand sides at once (mixed precision) ----------
@@ -621,6 +752,31 @@ __global__ void k_corrections(int nt, const int* __restrict__ toff, const int* _
     ys[nt + k] -= y2;
 }
 
+// Work items of the pair-tile kernel: the tiles (A, B), B a chunk of a neighbour leaf c2 >= leaf(A)
+// and B >= A, cut into items of n tiles that share A. An item costs its targets' load and two
+// FP64 atomics per lane, as much as a fraction of a tile; too few items leave the GPU's 152 x 24
+// warps idle at the end. n = 6 where every warp gets eight items or more, fewer below (81,920
+// elements: 72,000 tiles, n = 2: 178 -> 166 us; 1280: 820 tiles, n = 1: 27 -> 12 us).
+static void near_pair_items(int ncl, const std::vector<int>& first_chunk, const std::vector<int>& no,
+                            const std::vector<int>& ni, std::vector<int>& tl, std::vector<int4>& it)
+{
+    std::vector<int> start;  // first tile of each chunk
+    for (int k = 0; k < ncl; ++k)
+        for (int a = first_chunk[k]; a < first_chunk[k + 1]; ++a) {
+            start.push_back((int)tl.size());
+            for (int t = no[k]; t < no[k + 1]; ++t) {
+                const int c2 = ni[t];
+                if (c2 < k) continue;
+                for (int bq = (c2 == k ? a : first_chunk[c2]); bq < first_chunk[c2 + 1]; ++bq) tl.push_back(bq);
+            }
+        }
+    start.push_back((int)tl.size());
+    const int n = std::max(1, std::min(NEAR_ITEM, (int)(tl.size() / (152 * 24 * 8))));
+    for (size_t a = 0; a + 1 < start.size(); ++a)
+        for (int t = start[a]; t < start[a + 1]; t += n)
+            it.push_back(make_int4((int)a, t, std::min(t + n, start[a + 1]), 0));
+}
+
 // chunks of at most 32 targets per leaf and the packed source buffers (mixed precision)
 int pb_near_setup(pb_ctx* c)
 {
@@ -638,8 +794,6 @@ int pb_near_setup(pb_ctx* c)
             cf.push_back(s);
         }
     c->nchunks = (int)cl.size();
-    // pair tiles (A, B), B a chunk of a neighbour leaf c2 >= leaf(A) and B >= A, cut into work
-    // items of at most NEAR_ITEM tiles that share A
     {
         std::vector<int> first_chunk(lv.ncl + 1, 0);
         for (int k = 0; k < lv.ncl; ++k) first_chunk[k + 1] = first_chunk[k] + (b[k + 1] - b[k] + 31) / 32;
@@ -649,22 +803,7 @@ int pb_near_setup(pb_ctx* c)
         it.clear();
         const std::vector<int>& no = c->h_near_off;
         const std::vector<int>& ni = c->h_near_idx;
-        for (int k = 0; k < lv.ncl; ++k)
-            for (int a = first_chunk[k]; a < first_chunk[k + 1]; ++a) {
-                int start = (int)tl.size();
-                for (int t = no[k]; t < no[k + 1]; ++t) {
-                    const int c2 = ni[t];
-                    if (c2 < k) continue;
-                    for (int bq = (c2 == k ? a : first_chunk[c2]); bq < first_chunk[c2 + 1]; ++bq) {
-                        tl.push_back(bq);
-                        if ((int)tl.size() - start == NEAR_ITEM) {
-                            it.push_back(make_int4(a, start, (int)tl.size(), 0));
-                            start = (int)tl.size();
-                        }
-                    }
-                }
-                if ((int)tl.size() > start) it.push_back(make_int4(a, start, (int)tl.size(), 0));
-            }
+        near_pair_items(lv.ncl, first_chunk, no, ni, tl, it);
         c->near_nitems = (int)it.size();
         c->near_mitems = 0;  // the several-vector items are made on first use (pb_near_reserve)
         c->near_mitem = nullptr;
@@ -683,7 +822,8 @@ int pb_near_setup(pb_ctx* c)
         return pb_fail(c, PB_ERR_NOMEM, "near setup: out of memory");
     PB_CUDA(c, cudaMemcpyAsync(c->chunk_leaf, cl.data(), sizeof(int) * cl.size(), cudaMemcpyHostToDevice, c->st));
     PB_CUDA(c, cudaMemcpyAsync(c->chunk_first, cf.data(), sizeof(int) * cf.size(), cudaMemcpyHostToDevice, c->st));
-    return PB_OK;
+    return near_flags(c, c->nchunks, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p, c->near_nitems, c->near_items,
+                      c->near_tiles);
 }
 
 int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
@@ -695,7 +835,7 @@ int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
         k_near_pack<<<(nt + 255) / 256, 256, 0, c->st>>>(nt, c->e32p, c->e32n, xs, c->near_sp, c->near_sn);
         PB_LAUNCH(c);
         PB_CUDA(c, cudaMemsetAsync(ys, 0, sizeof(double) * 2 * nt, c->st));
-        k_near_tile<1><<<(c->near_nitems * 32 + 255) / 256, 256, 0, c->st>>>(
+        k_near_tile<1><<<(c->near_nitems + NEAR_W - 1) / NEAR_W, 32 * NEAR_W, 0, c->st>>>(
             nt, c->near_nitems, c->near_items, c->near_tiles, c->chunk_leaf, c->chunk_first, lv.begin, c->near_sp,
             c->near_sn, c->e32l, eps, c->prm.kappa, ys);
         PB_LAUNCH(c);
@@ -959,22 +1099,7 @@ int pb_near_points_setup(pb_ctx* c)
     }
     const std::vector<int>& no = c->h_near_off;
     const std::vector<int>& ni = c->h_near_idx;
-    for (int k = 0; k < lv.ncl; ++k)
-        for (int a = first_chunk[k]; a < first_chunk[k + 1]; ++a) {
-            int start = (int)tl.size();
-            for (int t = no[k]; t < no[k + 1]; ++t) {
-                const int c2 = ni[t];
-                if (c2 < k) continue;
-                for (int bq = (c2 == k ? a : first_chunk[c2]); bq < first_chunk[c2 + 1]; ++bq) {
-                    tl.push_back(bq);
-                    if ((int)tl.size() - start == NEAR_ITEM) {
-                        it.push_back(make_int4(a, start, (int)tl.size(), 0));
-                        start = (int)tl.size();
-                    }
-                }
-            }
-            if ((int)tl.size() > start) it.push_back(make_int4(a, start, (int)tl.size(), 0));
-        }
+    near_pair_items(lv.ncl, first_chunk, no, ni, tl, it);
     c->pn_nitems = (int)it.size();
     c->h_pn_i[0].swap(cl);
     c->h_pn_i[1].swap(cf);
@@ -1006,7 +1131,8 @@ int pb_near_points_setup(pb_ctx* c)
     PB_CUDA(c, cudaMemcpyAsync(c->pn_begin, c->begin_q, sizeof(int) * (lv.ncl + 1), cudaMemcpyDeviceToDevice, c->st));
     k_pts32<<<(unsigned)((np + 255) / 256), 256, 0, c->st>>>(np, c->pts_p, c->pts_n, c->pn_p32, c->pn_l32, c->pn_n32);
     PB_LAUNCH(c);
-    return PB_OK;
+    return near_flags(c, (int)c->h_pn_i[0].size(), c->pn_chunk_leaf, c->pn_chunk_first, c->pn_begin, c->pts_p,
+                      c->pn_nitems, c->pn_items, c->pn_tiles);
 }
 
 // ypt (2 np) = per point sum over the near points of other elements of K (W u), in FP64; the
@@ -1019,13 +1145,13 @@ int pb_near_points_apply(pb_ctx* c, const double* xs, const double* xq, double* 
                                                                  xq, c->pn_sp, c->pn_sn);
     PB_LAUNCH(c);
     PB_CUDA(c, cudaMemsetAsync(ypt, 0, sizeof(double) * 2 * np, c->st));
-    const unsigned nb = (unsigned)(((long long)c->pn_nitems * 32 + 255) / 256);
+    const unsigned nb = (unsigned)((c->pn_nitems + NEAR_W - 1) / NEAR_W);
     if (c->q2 == 4)
-        k_near_tile<4><<<nb, 256, 0, c->st>>>((int)np, c->pn_nitems, c->pn_items, c->pn_tiles, c->pn_chunk_leaf,
+        k_near_tile<4><<<nb, 32 * NEAR_W, 0, c->st>>>((int)np, c->pn_nitems, c->pn_items, c->pn_tiles, c->pn_chunk_leaf,
                                                c->pn_chunk_first, c->pn_begin, c->pn_sp, c->pn_sn, c->pn_l32, eps,
                                                c->prm.kappa, ypt);
     else
-        k_near_tile<16><<<nb, 256, 0, c->st>>>((int)np, c->pn_nitems, c->pn_items, c->pn_tiles, c->pn_chunk_leaf,
+        k_near_tile<16><<<nb, 32 * NEAR_W, 0, c->st>>>((int)np, c->pn_nitems, c->pn_items, c->pn_tiles, c->pn_chunk_leaf,
                                                 c->pn_chunk_first, c->pn_begin, c->pn_sp, c->pn_sn, c->pn_l32, eps,
                                                 c->prm.kappa, ypt);
     PB_LAUNCH(c);

@@ -336,3 +336,25 @@ def test_fp64_pair_tiles_ragged_leaves(leaf, levels, part):
         assert torch.equal(y, z)  # no atomics: the same product twice is the same bits
     finally:
         pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("kappa", [0.0, 0.02, KAP, 0.6, 3.0])
+@pytest.mark.parametrize("leaf,qr", [(1000, 0), (5, 0), (45, 0), (20, 2)])
+def test_mixed_near_tiles_against_fp64(kappa, leaf, qr):
+    # tiles within, across and beyond kappa r = 0.125 (where the screening series ends), full and
+    # remainder chunks on either side, points of a rule. Both runs hold the same FP64 corrections
+    # and mass terms, so what is left is the FP32 pair terms: about ten roundings of 6e-8 each
+    V, T = inputs.perturbed_sphere(3, 2.0, 0.2, seed=23)
+    m = inputs.Mesh(V, T[:1271], np.zeros((1, 3)), np.ones(1))
+    x = _dev(inputs.random_density(m.nt, 5))
+    got = []
+    for prec in (pb.PB_FP64, pb.PB_MIXED):
+        ctx = _ctx(m, kappa=kappa, eta0=0.8, leaf_size=leaf, p=4, qr=qr, precision=prec, precond=pb.PB_PRECOND_DIAG,
+                   singular=pb.PB_SINGULAR_FP64)
+        try:
+            y = torch.empty_like(x)
+            pb.pb_matvec_part(ctx, x, y, 1)
+            got.append(y.cpu().numpy())
+        finally:
+            pb.pb_destroy(ctx)
+    assert _rel(got[1], got[0]) < 6e-7
