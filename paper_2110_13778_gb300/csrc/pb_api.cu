@@ -144,6 +144,9 @@ extern "C" int pb_create(const pb_params* prm, void* stream, pb_ctx** out)
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (cudaStreamCreateWithPriority(&c->st2, cudaStreamNonBlocking, hi) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&c->st3, cudaStreamNonBlocking, hi) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_up, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_coarse, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_tree, cudaEventDisableTiming) != cudaSuccess ||
@@ -167,6 +170,12 @@ extern "C" int pb_destroy(pb_ctx* c)
         cudaStreamSynchronize(c->st2);
         cudaStreamDestroy(c->st2);
     }
+    if (c->st3) {
+        cudaStreamSynchronize(c->st3);
+        cudaStreamDestroy(c->st3);
+    }
+    if (c->ev_up) cudaEventDestroy(c->ev_up);
+    if (c->ev_coarse) cudaEventDestroy(c->ev_coarse);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->ev_tree) cudaEventDestroy(c->ev_tree);

@@ -62,7 +62,9 @@ struct pb_ctx {
     pb_params prm;
     cudaStream_t st = nullptr;
     cudaStream_t st2 = nullptr;      // far field, concurrent with the near field on st
+    cudaStream_t st3 = nullptr;      // far field: the coarser levels' upward pass and MtL
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_tree = nullptr;
+    cudaEvent_t ev_up = nullptr, ev_coarse = nullptr;
     cudaEvent_t ev_sing = nullptr;  // the singular pass has been queued up to here
     bool tables_ready = false;       // far-field constant tables uploaded
     std::string err = "no error";
