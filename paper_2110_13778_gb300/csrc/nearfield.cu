@@ -223,16 +223,27 @@ static int near64_setup(pb_ctx* c)
 
 // ---------- mixed precision near field ----------
 // Per matrix-vector product the sources are packed once as FP32 records
-// (x_hi, y_hi, z_hi, A phi), (n_x, n_y, n_z, A dphi) beside the fixed (x_lo, y_lo, z_lo).
+// (x_hi, y_hi, z_hi, A phi), (n_x, n_y, n_z, A dphi) beside the fixed (x_lo, y_lo, z_lo), and the
+// sums are set to zero. With order (the caller's vector is in element order) the tree-ordered copy
+// xs is made on the way.
 __global__ void k_near_pack(int nt, const float4* __restrict__ e32p, const float4* __restrict__ e32n,
-                            const double* __restrict__ xs, float4* __restrict__ sp, float4* __restrict__ sn)
+                            const int* __restrict__ order, const double* __restrict__ x, double* __restrict__ xs,
+                            float4* __restrict__ sp, float4* __restrict__ sn, double* __restrict__ ys)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nt) return;
     float4 p = e32p[k], n = e32n[k];
+    const int e = order ? order[k] : k;
+    const double v1 = x[e], v2 = x[nt + e];
+    if (order) {
+        xs[k] = v1;
+        xs[nt + k] = v2;
+    }
+    ys[k] = 0.0;
+    ys[nt + k] = 0.0;
     double A = (double)p.w;
-    sp[k] = make_float4(p.x, p.y, p.z, (float)(A * xs[k]));
-    sn[k] = make_float4(n.x, n.y, n.z, (float)(A * xs[nt + k]));
+    sp[k] = make_float4(p.x, p.y, p.z, (float)(A * v1));
+    sn[k] = make_float4(n.x, n.y, n.z, (float)(A * v2));
 }
 
 
@@ -613,14 +624,24 @@ static int near_flags(pb_ctx* c, int nchunks, const int* chunk_leaf, const int* 
 // The pair kernels depend on the geometry only, so one evaluation serves NR densities: the
 // source's geometry records are loaded once per pair and each right-hand side adds four FMAs.
 // dens[r nt + j] = (A_j phi_j, A_j dphi_j) of right-hand side r.
-__global__ void k_near_dens(int nt, const float4* __restrict__ e32p, const double* __restrict__ xs,
-                            float2* __restrict__ dens)
+// (and, as k_near_pack, the tree-ordered copy of an element-ordered vector and zero sums)
+__global__ void k_near_dens(int nt, const float4* __restrict__ e32p, const int* __restrict__ order,
+                            const double* __restrict__ x, double* __restrict__ xs, float2* __restrict__ dens,
+                            double* __restrict__ ys)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nt) return;
     const double A = (double)e32p[k].w;
-    const double* x = xs + 2LL * nt * blockIdx.y;
-    dens[(size_t)nt * blockIdx.y + k] = make_float2((float)(A * x[k]), (float)(A * x[nt + k]));
+    const long long o = 2LL * nt * blockIdx.y;
+    const int e = order ? order[k] : k;
+    const double v1 = x[o + e], v2 = x[o + nt + e];
+    if (order) {
+        xs[o + k] = v1;
+        xs[o + nt + k] = v2;
+    }
+    ys[o + k] = 0.0;
+    ys[o + nt + k] = 0.0;
+    dens[(size_t)nt * blockIdx.y + k] = make_float2((float)(A * v1), (float)(A * v2));
 }
 
 // Work items of at most NEAR_ITEM_M directed tiles (target chunk A, source chunk B of any
@@ -708,48 +729,80 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
             }
 }
 
-// y1 = 1/2 (1 + eps) A phi - A acc1, y2 = 1/2 (1 + 1/eps) A dphi - A acc2 (FP64)
-__global__ void k_near_finish(int nt, const double4_32a* __restrict__ ep, const double* __restrict__ xs,
-                              double eps, double* __restrict__ ys)
+// What ends a product. ep: ys holds the mixed near field's bare sums, which become
+// y1 = 1/2 (1 + eps) A phi - A acc1, y2 = 1/2 (1 + 1/eps) A dphi - A acc2 (nullptr: ys holds rows);
+// yf: the far-field part to add (or nullptr); order: the result goes to y[order[k]] in element
+// order, else to y[k] in tree order.
+struct MvEnd {
+    int nt;
+    const double4_32a* ep;
+    double eps;
+    const double *xs, *ys, *yf;
+    const int* order;
+    double* y;
+};
+__device__ __forceinline__ void mv_end(const MvEnd& m, long long o, int k, double c1, double c2)
 {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nt) return;
-    xs += 2LL * nt * blockIdx.y;
-    ys += 2LL * nt * blockIdx.y;
-    double A = ep[k].w;
-    ys[k] = 0.5 * (1.0 + eps) * A * xs[k] - A * ys[k];
-    ys[nt + k] = 0.5 * (1.0 + 1.0 / eps) * A * xs[nt + k] - A * ys[nt + k];
+    double a = m.ys[o + k], b = m.ys[o + m.nt + k];
+    if (m.ep) {
+        const double A = m.ep[k].w;
+        a = 0.5 * (1.0 + m.eps) * A * m.xs[o + k] - A * a;
+        b = 0.5 * (1.0 + 1.0 / m.eps) * A * m.xs[o + m.nt + k] - A * b;
+    }
+    if (m.yf) {
+        c1 -= m.yf[o + k];
+        c2 -= m.yf[o + m.nt + k];
+    }
+    const int e = m.order ? m.order[k] : k;
+    m.y[o + e] = a - c1;
+    m.y[o + m.nt + e] = b - c2;
 }
 
-// Sauter-Schwab corrections of identical and adjacent pairs (FP64), and the far-field part of
-// the product when yf is given (xs == nullptr: the far field alone)
-__global__ void k_corrections(int nt, const int* __restrict__ toff, const int* __restrict__ tj,
-                              const double* __restrict__ corr, const double* __restrict__ xs,
-                              double* __restrict__ ys, const double* __restrict__ yf)
+// Sauter-Schwab corrections of identical and adjacent pairs (FP64), and the end of the product.
+// One warp per 32 rows: their pairs (about 13 per row, one after the other in memory) are read as one
+// coalesced stream, 512 at a time with all loads independent, the products go through shared
+// memory and each lane adds its own row in order. Bound: the 36 bytes per pair from HBM (or
+// L2). A thread that walked its own row took 14 us on 1280 elements, 24.5 on 81,920 and 124 on
+// 737,280 (3.3 TB/s), the end of the product 4, 6 and 24 more; now 12, 24 and 142 us for
+// both (the FP64 pipe is a bound too: six operations per pair, 93 us at 737,280).
+#define CORR_W 4
+#define CORR_B 512
+__global__ void __launch_bounds__(32 * CORR_W) k_corrections(const int* __restrict__ toff, const int* __restrict__ tj,
+                                                             const double* __restrict__ corr, MvEnd m)
 {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nt) return;
-    const long long o = 2LL * nt * blockIdx.y;
-    ys += o;
+    __shared__ double s1[CORR_W][CORR_B], s2[CORR_W][CORR_B];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt = m.nt;
+    const int k0 = (blockIdx.x * CORR_W + w) * 32, k = k0 + lane;
+    if (k0 >= nt) return;
+    const int t0 = toff[min(k, nt)], t1 = toff[min(k + 1, nt)];
+    const int e0 = __shfl_sync(0xffffffffu, t0, 0), e1 = __shfl_sync(0xffffffffu, t1, 31);
+    const double2* c2 = reinterpret_cast<const double2*>(corr);
     double y1 = 0.0, y2 = 0.0;
-    if (xs) {
-        xs += o;
-        // the four values of a pair as two 16-byte loads
-        const double2* c2 = reinterpret_cast<const double2*>(corr);
-        for (int t = toff[k]; t < toff[k + 1]; ++t) {
-            int j = tj[t];
-            double ph = xs[j], dph = xs[nt + j];
-            const double2 a = c2[2 * t], b = c2[2 * t + 1];
-            y1 += a.x * dph + a.y * ph;
-            y2 += b.x * dph + b.y * ph;
+    for (int base = e0; base < e1; base += CORR_B) {
+        const int n = min(CORR_B, e1 - base);
+#pragma unroll 4
+        for (int i = lane; i < n; i += 32) {
+            const int t = base + i, j = tj[t];
+            const double2 a = c2[2 * (size_t)t], b = c2[2 * (size_t)t + 1];
+            const double ph = m.xs[j], dph = m.xs[nt + j];
+            s1[w][i] = a.x * dph + a.y * ph;
+            s2[w][i] = b.x * dph + b.y * ph;
         }
+        __syncwarp();
+        for (int i = max(t0 - base, 0); i < min(t1 - base, n); ++i) {
+            y1 += s1[w][i];
+            y2 += s2[w][i];
+        }
+        __syncwarp();
     }
-    if (yf) {
-        y1 -= yf[o + k];
-        y2 -= yf[o + nt + k];
-    }
-    ys[k] -= y1;
-    ys[nt + k] -= y2;
+    if (k < nt) mv_end(m, 0, k, y1, y2);
+}
+
+// the far-field part alone, for any number of vectors
+__global__ void k_mv_end(MvEnd m)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < m.nt) mv_end(m, 2LL * m.nt * blockIdx.y, k, 0.0, 0.0);
 }
 
 // Work items of the pair-tile kernel: the tiles (A, B), B a chunk of a neighbour leaf c2 >= leaf(A)
@@ -826,20 +879,33 @@ int pb_near_setup(pb_ctx* c)
                       c->near_tiles);
 }
 
+// Mixed precision, one-point rule: before the near field of nr vectors, the packed densities and
+// zero sums; xin: the vectors in element order (xs is then written), or nullptr.
+int pb_near_pack(pb_ctx* c, const double* xin, double* xs, double* ys, int nr)
+{
+    const int nt = c->nt;
+    const int* order = xin ? c->order : nullptr;
+    const double* x = xin ? xin : xs;
+    if (nr == 1) {
+        k_near_pack<<<(nt + 255) / 256, 256, 0, c->st>>>(nt, c->e32p, c->e32n, order, x, xs, c->near_sp, c->near_sn, ys);
+    } else {
+        int rc = pb_near_reserve(c, nr);
+        if (rc) return rc;
+        k_near_dens<<<dim3((nt + 255) / 256, nr), 256, 0, c->st>>>(nt, c->e32p, order, x, xs, c->near_dens, ys);
+    }
+    PB_LAUNCH(c);
+    return PB_OK;
+}
+
+// one vector; mixed: adds the bare sums into ys (after pb_near_pack), FP64: writes the rows
 int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
 {
     const PbLevel& lv = c->lev[c->L];
     double eps = c->prm.eps_out / c->prm.eps_in;
     if (c->prm.precision == PB_MIXED) {
-        const int nt = c->nt;
-        k_near_pack<<<(nt + 255) / 256, 256, 0, c->st>>>(nt, c->e32p, c->e32n, xs, c->near_sp, c->near_sn);
-        PB_LAUNCH(c);
-        PB_CUDA(c, cudaMemsetAsync(ys, 0, sizeof(double) * 2 * nt, c->st));
         k_near_tile<1><<<(c->near_nitems + NEAR_W - 1) / NEAR_W, 32 * NEAR_W, 0, c->st>>>(
-            nt, c->near_nitems, c->near_items, c->near_tiles, c->chunk_leaf, c->chunk_first, lv.begin, c->near_sp,
+            c->nt, c->near_nitems, c->near_items, c->near_tiles, c->chunk_leaf, c->chunk_first, lv.begin, c->near_sp,
             c->near_sn, c->e32l, eps, c->prm.kappa, ys);
-        PB_LAUNCH(c);
-        k_near_finish<<<(nt + 255) / 256, 256, 0, c->st>>>(nt, c->e64p, xs, eps, ys);
     } else {
         k_near64<<<(unsigned)(((long long)c->near_nitems * 32 + 255) / 256), 256, 0, c->st>>>(
             c->nt, c->near_nitems, c->near_tiles2, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p, c->e64n, xs, eps,
@@ -855,54 +921,49 @@ int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
 
 // Several right-hand sides: four per thread (blockIdx.y = group of four), so each correction
 // is read once per four vectors instead of once per vector.
-__global__ void k_corrections4(int nt, int nr, const int* __restrict__ toff, const int* __restrict__ tj,
-                               const double* __restrict__ corr, const double* __restrict__ xs,
-                               double* __restrict__ ys, const double* __restrict__ yf)
+__global__ void k_corrections4(int nr, const int* __restrict__ toff, const int* __restrict__ tj,
+                               const double* __restrict__ corr, MvEnd m)
 {
+    const int nt = m.nt;
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nt) return;
     const int q0 = 4 * blockIdx.y, nq = min(4, nr - q0);
     const long long vs = 2LL * nt;
     double y1[4] = {0, 0, 0, 0}, y2[4] = {0, 0, 0, 0};
-    if (xs)
-        for (int t = toff[k]; t < toff[k + 1]; ++t) {
-            const int j = tj[t];
-            const double2 a = reinterpret_cast<const double2*>(corr)[2 * t];
-            const double2 b = reinterpret_cast<const double2*>(corr)[2 * t + 1];
-            const double c0 = a.x, c1 = a.y, c2 = b.x, c3 = b.y;
+    for (int t = toff[k]; t < toff[k + 1]; ++t) {
+        const int j = tj[t];
+        const double2 a = reinterpret_cast<const double2*>(corr)[2 * t];
+        const double2 b = reinterpret_cast<const double2*>(corr)[2 * t + 1];
+        const double c0 = a.x, c1 = a.y, c2 = b.x, c3 = b.y;
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < nq) {
-                    const double* x = xs + (q0 + q) * vs;
-                    const double ph = x[j], dph = x[nt + j];
-                    y1[q] += c0 * dph + c1 * ph;
-                    y2[q] += c2 * dph + c3 * ph;
-                }
-        }
+        for (int q = 0; q < 4; ++q)
+            if (q < nq) {
+                const double* x = m.xs + (q0 + q) * vs;
+                const double ph = x[j], dph = x[nt + j];
+                y1[q] += c0 * dph + c1 * ph;
+                y2[q] += c2 * dph + c3 * ph;
+            }
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-        if (q < nq) {
-            const long long o = (q0 + q) * vs;
-            double a = y1[q], b = y2[q];
-            if (yf) {
-                a -= yf[o + k];
-                b -= yf[o + nt + k];
-            }
-            ys[o + k] -= a;
-            ys[o + nt + k] -= b;
-        }
+        if (q < nq) mv_end(m, (q0 + q) * vs, k, y1[q], y2[q]);
 }
 
-int pb_corr_apply(pb_ctx* c, const double* xs, double* ys, int nr, const double* yfar)
+// corrections (with xs; without: the far field alone), far-field part and end of the product of nr
+// vectors into y: in element order, or in tree order. sums: ys holds bare near-field sums.
+int pb_corr_apply(pb_ctx* c, const double* xs, const double* ys, int nr, const double* yfar, bool sums, bool element_order,
+                  double* y)
 {
-    if (nr > 1) {
-        k_corrections4<<<dim3((c->nt + 255) / 256, (nr + 3) / 4), 256, 0, c->st>>>(c->nt, nr, c->touch_off, c->touch_j,
-                                                                                c->corr, xs, ys, yfar);
-        PB_LAUNCH(c);
-        return PB_OK;
-    }
-    k_corrections<<<dim3((c->nt + 255) / 256, nr), 256, 0, c->st>>>(c->nt, c->touch_off, c->touch_j, c->corr, xs,
-                                                                     ys, yfar);
+    const int nt = c->nt;
+    const MvEnd m = {nt, sums ? c->e64p : nullptr, c->prm.eps_out / c->prm.eps_in, xs, ys, yfar,
+                     element_order ? c->order : nullptr, y};
+    if (!xs)
+        k_mv_end<<<dim3((nt + 255) / 256, nr), 256, 0, c->st>>>(m);
+    else if (nr > 1)
+        k_corrections4<<<dim3((nt + 255) / 256, (nr + 3) / 4), 256, 0, c->st>>>(nr, c->touch_off, c->touch_j, c->corr, m);
+    else
+        k_corrections<<<(nt + 32 * CORR_W - 1) / (32 * CORR_W), 32 * CORR_W, 0, c->st>>>(c->touch_off, c->touch_j, c->corr,
+                                                                                        m);
     PB_LAUNCH(c);
     return PB_OK;
 }
@@ -979,8 +1040,8 @@ int pb_near_reserve(pb_ctx* c, int nr)
     return PB_OK;
 }
 
-// nr right-hand sides: xs and ys hold nr vectors of 2 nt; mixed precision evaluates each pair
-// once for up to 16 of them, FP64 applies the single-vector kernel per right-hand side
+// nr right-hand sides: xs and ys hold nr vectors of 2 nt (mixed: bare sums, after pb_near_pack); mixed
+// precision evaluates each pair once for up to 16 of them, FP64 applies the single-vector kernel per right-hand side
 int pb_near_apply_multi(pb_ctx* c, const double* xs, double* ys, int nr)
 {
     const int nt = c->nt;
@@ -992,11 +1053,6 @@ int pb_near_apply_multi(pb_ctx* c, const double* xs, double* ys, int nr)
         }
         return PB_OK;
     }
-    int rc0 = pb_near_reserve(c, nr);
-    if (rc0) return rc0;
-    k_near_dens<<<dim3((nt + 255) / 256, nr), 256, 0, c->st>>>(nt, c->e32p, xs, c->near_dens);
-    PB_LAUNCH(c);
-    PB_CUDA(c, cudaMemsetAsync(ys, 0, sizeof(double) * 2 * (size_t)nt * nr, c->st));
     // groups of up to 16 right-hand sides, each one launch of the smallest width that holds it
     // (the density buffer is padded to a multiple of 16 vectors)
     for (int r0 = 0; r0 < nr;) {
@@ -1012,8 +1068,6 @@ int pb_near_apply_multi(pb_ctx* c, const double* xs, double* ys, int nr)
         if (rc) return rc;
         r0 += v;
     }
-    k_near_finish<<<dim3((nt + 255) / 256, nr), 256, 0, c->st>>>(nt, c->e64p, xs, eps, ys);
-    PB_LAUNCH(c);
     return PB_OK;
 }
 

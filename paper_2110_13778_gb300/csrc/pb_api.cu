@@ -381,36 +381,50 @@ void pb_drop_graphs(pb_ctx* c)
     c->gb_graph_key = nullptr;
 }
 
-static int matvec_parts(pb_ctx* c, const double* xs, double* ys, int nr, int which)
+// xin: the vectors in element order (xs, a work vector of the context, is then filled from them), or
+// nullptr; y: the result, in element order if xin is given, else in tree order; ys: work vector
+// (may be y when xin is nullptr).
+static int matvec_parts(pb_ctx* c, const double* xin, double* xs, double* ys, double* y, int nr, int which)
 {
     int rc;
+    const int n = c->nt;
     if (c->q2 > 1 && nr > 1) {  // the regular rule of order > 1 works one vector at a time
-        for (int r = 0; r < nr; ++r)
-            if ((rc = matvec_parts(c, xs + 2LL * c->nt * r, ys + 2LL * c->nt * r, 1, which))) return rc;
+        for (int r = 0; r < nr; ++r) {
+            const long long o = 2LL * n * r;
+            if ((rc = matvec_parts(c, xin ? xin + o : nullptr, xs + o, ys + o, y + o, 1, which))) return rc;
+        }
         return PB_OK;
     }
-    const bool far = which != 1;
+    const bool far = which != 1, near = which != 2;
+    const bool sums = near && c->prm.precision == PB_MIXED && c->q2 == 1;  // the near field leaves bare sums
     // every buffer the product touches exists before the fork (and before any capture)
     if ((rc = pb_matvec_reserve(c, nr))) return rc;
+    if (xin && sums) {
+        if ((rc = pb_near_pack(c, xin, xs, ys, nr))) return rc;
+    } else if (xin) {
+        k_gather<<<dim3((n + 255) / 256, nr), 256, 0, c->st>>>(n, c->order, xin, xs);
+        PB_LAUNCH(c);
+    }
     if (far) {
         PB_CUDA(c, cudaEventRecord(c->ev_fork, c->st));
         PB_CUDA(c, cudaStreamWaitEvent(c->st2, c->ev_fork, 0));
         if ((rc = pb_far_apply(c, xs, c->yfar, nr, c->st2))) return rc;
         PB_CUDA(c, cudaEventRecord(c->ev_join, c->st2));
     }
-    if (which == 2) {
+    if (!near) {
         PB_CUDA(c, cudaMemsetAsync(ys, 0, sizeof(double) * 2 * c->nt * nr, c->st));
         PB_CUDA(c, cudaStreamWaitEvent(c->st, c->ev_join, 0));
-        return pb_corr_apply(c, nullptr, ys, nr, c->yfar);
+        return pb_corr_apply(c, nullptr, ys, nr, c->yfar, false, xin != nullptr, y);
     }
     pb_tic(c, PB_T_NEAR);
+    if (!xin && sums && (rc = pb_near_pack(c, nullptr, xs, ys, nr))) return rc;
     if ((rc = c->q2 > 1 ? pb_near_q_apply(c, xs, ys)
                         : nr == 1 ? pb_near_apply(c, xs, ys) : pb_near_apply_multi(c, xs, ys, nr)))
         return rc;
     pb_toc(c, PB_T_NEAR);
     if (far) PB_CUDA(c, cudaStreamWaitEvent(c->st, c->ev_join, 0));
     pb_tic(c, PB_T_CORR);
-    if ((rc = pb_corr_apply(c, xs, ys, nr, far ? c->yfar : nullptr))) return rc;
+    if ((rc = pb_corr_apply(c, xs, ys, nr, far ? c->yfar : nullptr, sums, xin != nullptr, y))) return rc;
     pb_toc(c, PB_T_CORR);
     return PB_OK;
 }
@@ -418,7 +432,7 @@ static int matvec_parts(pb_ctx* c, const double* xs, double* ys, int nr, int whi
 int pb_matvec_sorted(pb_ctx* c, const double* xs, double* ys, int which)
 {
     if (c->prm.basis == PB_BASIS_LINEAR) return pb_p1_matvec(c, xs, ys);
-    return matvec_parts(c, xs, ys, 1, which);
+    return matvec_parts(c, nullptr, const_cast<double*>(xs), ys, ys, 1, which);  // (xs is only read without xin)
 }
 
 // nr products at once: xs and ys hold nr vectors of 2 nt in tree order
@@ -428,7 +442,7 @@ int pb_matvec_sorted_multi(pb_ctx* c, const double* xs, double* ys, int nr)
         if (nr != 1) return pb_fail(c, PB_ERR_ARG, "piecewise-linear basis: one vector at a time");
         return pb_p1_matvec(c, xs, ys);
     }
-    return matvec_parts(c, xs, ys, nr, 0);
+    return matvec_parts(c, nullptr, const_cast<double*>(xs), ys, ys, nr, 0);
 }
 
 // tree-ordered work vectors for nr right-hand sides (build lifetime, grown on demand)
@@ -451,13 +465,7 @@ extern "C" int pb_matvec_multi(pb_ctx* c, const double* X, double* Y, int nr)
     if (c->prm.basis != PB_BASIS_CONSTANT) return pb_fail(c, PB_ERR_ARG, "matvec_multi: piecewise-constant basis only");
     int rc;
     if ((rc = reserve_multi(c, nr))) return rc;
-    const int n = c->nt;
-    k_gather<<<dim3((n + 255) / 256, nr), 256, 0, c->st>>>(n, c->order, X, c->mxs);
-    PB_LAUNCH(c);
-    if ((rc = pb_matvec_sorted_multi(c, c->mxs, c->mys, nr))) return rc;
-    k_scatter<<<dim3((n + 255) / 256, nr), 256, 0, c->st>>>(n, c->order, c->mys, Y);
-    PB_LAUNCH(c);
-    return PB_OK;
+    return matvec_parts(c, X, c->mxs, c->mys, Y, nr, 0);
 }
 
 extern "C" int pb_matvec_part(pb_ctx* c, const double* x, double* y, int which)
@@ -467,6 +475,7 @@ extern "C" int pb_matvec_part(pb_ctx* c, const double* x, double* y, int which)
     if (!x || !y || x == y || which < 0 || which > 2) return pb_fail(c, PB_ERR_ARG, "matvec: bad arguments");
     if (which != 0 && c->prm.basis != PB_BASIS_CONSTANT)
         return pb_fail(c, PB_ERR_ARG, "matvec_part: piecewise-constant basis only");
+    if (c->prm.basis == PB_BASIS_CONSTANT) return matvec_parts(c, x, c->xs, c->ys, y, 1, which);
     int rc;
     if ((rc = pb_gather(c, x, c->xs))) return rc;
     if ((rc = pb_matvec_sorted(c, c->xs, c->ys, which))) return rc;

@@ -287,9 +287,11 @@ int pb_scan_exclusive(pb_ctx* c, const int* in, int* out, int n);
 int pb_radix_sort_pairs(pb_ctx* c, const unsigned* kin, const int* vin, unsigned* kout, int* vout, int n, int bits);
 int pb_touching_and_singular(pb_ctx* c);      // singular.cu
 int pb_near_setup(pb_ctx* c);                                      // nearfield.cu
-int pb_near_apply(pb_ctx* c, const double* xs, double* ys);        // nearfield.cu (writes ys)
-int pb_corr_apply(pb_ctx* c, const double* xs, double* ys, int nr, const double* yfar);  // nearfield.cu (adds)
-int pb_near_apply_multi(pb_ctx* c, const double* xs, double* ys, int nr);  // nearfield.cu (writes)
+int pb_near_pack(pb_ctx* c, const double* xin, double* xs, double* ys, int nr);  // nearfield.cu (mixed, one-point rule)
+int pb_near_apply(pb_ctx* c, const double* xs, double* ys);                 // nearfield.cu
+int pb_near_apply_multi(pb_ctx* c, const double* xs, double* ys, int nr);   // nearfield.cu
+int pb_corr_apply(pb_ctx* c, const double* xs, const double* ys, int nr, const double* yfar, bool sums, bool element_order,
+                  double* y);  // nearfield.cu
 int pb_near_reserve(pb_ctx* c, int nr);
 int pb_far_setup(pb_ctx* c);                                       // farfield.cu
 int pb_far_apply(pb_ctx* c, const double* xs, double* ys, int nr, cudaStream_t st);  // farfield.cu (sets ys)
