@@ -61,19 +61,42 @@ __device__ __forceinline__ void pb_screen<double>(double t, double& E, double& g
     g = E + t;
 }
 
+// The bare instructions, which flush subnormal numbers: the bits of rsqrtf and of __expf's exponential
+// wherever the argument (the result) is a normal number.
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // K[0..3] = K1..K4 for d = x - y, target normal n_x, source normal n_y, all scaled by `scale`
 // (0 drops a pair without extra products: it multiplies 1 / (4 pi r), which every term carries).
-template <class R>
+// FAR (FP32): the caller knows that t >= 0.125, where the series of pb_screen is not chosen.
+template <class R, bool FAR = false>
 __device__ __forceinline__ void pb_kernels(R dx, R dy, R dz, R nxx, R nxy, R nxz, R nyx, R nyy, R nyz,
                                            R eps, R inv_eps, R kappa, R* K, R scale = R(1))
 {
     const R i4pi = R(0.07957747154594767) * scale;  // 1 / (4 pi), scaled
     R r2 = dx * dx + dy * dy + dz * dz;
-    R rinv = PbKer<R>::rsqrt_(r2);
+    R rinv;
+    if constexpr (FAR) rinv = rsqrt_ftz(r2);
+    else rinv = PbKer<R>::rsqrt_(r2);
     R r = r2 * rinv;
     R t = kappa * r;
     R E, g;
-    pb_screen<R>(t, E, g);
+    if constexpr (FAR) {
+        E = ex2_ftz(t * -1.4426950408889634f) - 1.0f;
+        g = E + t;
+    } else {
+        pb_screen<R>(t, E, g);
+    }
     R tE = t * E;
     R c1 = -g - tE;
     R c3 = R(-3) * g - t * t - tE * (R(3) + t);

@@ -281,19 +281,6 @@ __global__ void k_near_pack(int nt, const float4* __restrict__ e32p, const float
 // function in every tile: 3090 -> 2567 us there, 202 -> 158 us on 81,920 elements (leaves of 71:
 // 20 % of the steps are remainder tiles), 35 -> 12 us on 1280. Blocks of four warps, because items
 // differ in length; seven per SM (72 registers) is the best of 5 to 8 by 1 to 4 %.
-__device__ __forceinline__ float rsqrt_ftz(float x)
-{
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float ex2_ftz(float x)
-{
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 struct NearTgt2 {
     f2x px, py, pz, lx, ly, lz, nx, ny, nz, phi, dphi;
 };
@@ -648,7 +635,53 @@ __global__ void k_near_dens(int nt, const float4* __restrict__ e32p, const int* 
 // neighbour leaf), one warp each; the item's sums are added into ys (zeroed first) with FP64
 // atomics, so that items of one target chunk may run on different warps. Each tile's source
 // records and its NR densities are staged in shared memory by coalesced loads (one per lane
-// and record), so the pair loop reads them as shared-memory broadcasts.
+// and record), so the pair loop reads them as shared-memory broadcasts. Two densities (r, r + 1) are
+// the halves of packed FP32 pairs in the four FMAs per density. A tile's FP32 sums go into
+// float-float accumulators (an exact two-sum, 2^-48): with FP64 ones (a conversion and an addition per
+// value, at 1/64 of the FP32 rate) the FP64 pipe was 55 % busy and held the loop up. 81,920 elements,
+// 16 densities: 870 -> 635 us.
+template <int NR>
+struct NearM {
+    static constexpr int H = (NR + 1) / 2;  // pairs of densities
+    static constexpr size_t smem = 8 * 32 * (3 * sizeof(float4) + H * sizeof(float4) + 4 * H * sizeof(f2x));
+};
+
+// the pairs of one tile: s1, s2 += per density pair
+template <int NR, bool FAR>
+__device__ __forceinline__ void near_m_tile(const float4 tp, const float4 tn, const float4 tl,
+                                            const float4* __restrict__ s_p, const float4* __restrict__ s_n,
+                                            const float4* __restrict__ s_l, const float4* __restrict__ s_d, int nb, int self,
+                                            float eps, float inv_eps, float kappa, f2x* s1, f2x* s2)
+{
+#pragma unroll 2
+    for (int q = 0; q < nb; ++q) {
+        const float4 a = s_p[q], b = s_n[q], l = s_l[q];
+        float K[4];
+        float dx = (tp.x - a.x) + (tl.x - l.x);
+        float dy = (tp.y - a.y) + (tl.y - l.y);
+        float dz = (tp.z - a.z) + (tl.z - l.z);
+        if (!FAR && q == self) dx = 1.0f;  // the identical pair is the correction's; keep r finite
+        pb_kernels<float, FAR>(dx, dy, dz, tn.x, tn.y, tn.z, b.x, b.y, b.z, eps, inv_eps, kappa, K,
+                               (!FAR && q == self) ? 0.f : 1.f);
+        const f2x k0 = x2_dup(K[0]), k1 = x2_dup(K[1]), k2 = x2_dup(K[2]), k3 = x2_dup(K[3]);
+#pragma unroll
+        for (int h = 0; h < NearM<NR>::H; ++h) {
+            const float4 d = s_d[h * 32 + q];
+            const f2x x = x2_pack(d.x, d.y), y = x2_pack(d.z, d.w);
+            s1[h] = x2_fma(k0, y, x2_fma(k1, x, s1[h]));
+            s2[h] = x2_fma(k2, y, x2_fma(k3, x, s2[h]));
+        }
+    }
+}
+
+// (hi, lo) += s, per half
+__device__ __forceinline__ void x2_ff_acc(f2x& hi, f2x& lo, f2x s)
+{
+    const f2x t = x2_add(hi, s), bb = x2_sub(t, hi);
+    lo = x2_add(lo, x2_add(x2_sub(hi, x2_sub(t, bb)), x2_sub(s, bb)));
+    hi = t;
+}
+
 template <int NR>
 __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const int4* __restrict__ items,
                                                     const int* __restrict__ tiles, const int* __restrict__ chunk_leaf,
@@ -658,16 +691,17 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
                                                     const float2* __restrict__ dens, double eps_d, double kappa_d,
                                                     double* __restrict__ ys, int nvalid)
 {
-    // dynamic shared memory (near32m_smem<NR>()): per warp the tile's source records, its NR
-    // densities, and the item's FP64 sums (kept here rather than in registers)
+    // dynamic shared memory: per warp the tile's source records, its densities in pairs, and the
+    // item's float-float sums (kept here rather than in registers)
+    constexpr int H = NearM<NR>::H;
     extern __shared__ __align__(16) unsigned char nsm[];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     float4* s_p = (float4*)nsm + wi * 32;
     float4* s_n = (float4*)nsm + 256 + wi * 32;
     float4* s_l = (float4*)nsm + 512 + wi * 32;
-    float2* s_d = (float2*)((float4*)nsm + 768) + wi * NR * 32;
-    double* s_acc = (double*)((float2*)((float4*)nsm + 768) + 8 * NR * 32) + wi * 2 * NR * 32;
+    float4* s_d = (float4*)nsm + 768 + wi * H * 32;                           // (x_r, x_r+1, y_r, y_r+1)
+    f2x* s_acc = (f2x*)((float4*)nsm + 768 + 8 * H * 32) + wi * 4 * H * 32;  // [4 h + (hi1, lo1, hi2, lo2)][lane]
     if (w >= nitems) return;
     const int4 item = items[w];
     const int c = chunk_leaf[item.x];
@@ -677,9 +711,9 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
     const float4 tp = sp[kk], tn = sn[kk], tl = sl[kk];
     const float eps = (float)eps_d, inv_eps = (float)(1.0 / eps_d), kappa = (float)kappa_d;
 #pragma unroll
-    for (int r = 0; r < 2 * NR; ++r) s_acc[r * 32 + lane] = 0.0;
+    for (int r = 0; r < 4 * H; ++r) s_acc[r * 32 + lane] = 0ull;
     for (int ti = item.y; ti < item.z; ++ti) {
-        const int cb = tiles[ti];
+        const int tv = tiles[ti], cb = tv & (NEAR_FAR - 1);
         const int sb = chunk_first[cb], se = min(sb + 32, begin[chunk_leaf[cb] + 1]);
         const int nb = se - sb;
         __syncwarp();
@@ -689,44 +723,44 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
             s_n[lane] = sn[j];
             s_l[lane] = sl[j];
 #pragma unroll
-            for (int r = 0; r < NR; ++r) s_d[r * 32 + lane] = dens[(size_t)nt * r + j];
-        }
-        __syncwarp();
-        float s1[NR], s2[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) s1[r] = s2[r] = 0.f;
-#pragma unroll 2
-        for (int q = 0; q < nb; ++q) {
-            const int j = sb + q;
-            const float4 a = s_p[q], b = s_n[q], l = s_l[q];
-            float K[4];
-            float dx = (tp.x - a.x) + (tl.x - l.x);
-            float dy = (tp.y - a.y) + (tl.y - l.y);
-            float dz = (tp.z - a.z) + (tl.z - l.z);
-            if (j == k) dx = 1.0f;  // the identical pair is the correction's; keep r finite
-            pb_kernels<float>(dx, dy, dz, tn.x, tn.y, tn.z, b.x, b.y, b.z, eps, inv_eps, kappa, K,
-                              (j == k) ? 0.f : 1.f);
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const float2 d = s_d[r * 32 + q];
-                s1[r] = fmaf(K[0], d.y, fmaf(K[1], d.x, s1[r]));
-                s2[r] = fmaf(K[2], d.y, fmaf(K[3], d.x, s2[r]));
+            for (int h = 0; h < H; ++h) {
+                const float2 d0 = dens[(size_t)nt * (2 * h) + j];
+                const float2 d1 = NR > 1 ? dens[(size_t)nt * (2 * h + 1) + j] : make_float2(0.f, 0.f);
+                s_d[h * 32 + lane] = make_float4(d0.x, d1.x, d0.y, d1.y);
             }
         }
+        __syncwarp();
+        f2x s1[H], s2[H];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            s_acc[r * 32 + lane] += (double)s1[r];
-            s_acc[(NR + r) * 32 + lane] += (double)s2[r];
+        for (int h = 0; h < H; ++h) s1[h] = s2[h] = 0ull;
+        if (tv & NEAR_FAR) near_m_tile<NR, true>(tp, tn, tl, s_p, s_n, s_l, s_d, nb, -1, eps, inv_eps, kappa, s1, s2);
+        else near_m_tile<NR, false>(tp, tn, tl, s_p, s_n, s_l, s_d, nb, k - sb, eps, inv_eps, kappa, s1, s2);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            f2x* a = s_acc + 4 * h * 32 + lane;
+            x2_ff_acc(a[0], a[32], s1[h]);
+            x2_ff_acc(a[64], a[96], s2[h]);
         }
     }
     // densities beyond nvalid are padding of the group (finite, unused): only nvalid are added
     if (act)
 #pragma unroll
-        for (int r = 0; r < NR; ++r)
-            if (r < nvalid) {
-                atomicAdd(&ys[2LL * nt * r + k], s_acc[r * 32 + lane]);
-                atomicAdd(&ys[2LL * nt * r + nt + k], s_acc[(NR + r) * 32 + lane]);
+        for (int h = 0; h < H; ++h) {
+            const f2x* a = s_acc + 4 * h * 32 + lane;
+            float h1[2], l1[2], h2[2], l2[2];
+            x2_unpack(a[0], h1[0], h1[1]);
+            x2_unpack(a[32], l1[0], l1[1]);
+            x2_unpack(a[64], h2[0], h2[1]);
+            x2_unpack(a[96], l2[0], l2[1]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int r = 2 * h + u;
+                if (r < nvalid) {
+                    atomicAdd(&ys[2LL * nt * r + k], (double)h1[u] + (double)l1[u]);
+                    atomicAdd(&ys[2LL * nt * r + nt + k], (double)h2[u] + (double)l2[u]);
+                }
             }
+        }
 }
 
 // What ends a product. ep: ys holds the mixed near field's bare sums, which become
@@ -969,18 +1003,12 @@ int pb_corr_apply(pb_ctx* c, const double* xs, const double* ys, int nr, const d
 }
 
 template <int NR>
-static constexpr size_t near32m_smem()
-{
-    return 768 * sizeof(float4) + 8 * NR * 32 * sizeof(float2) + 8 * 2 * NR * 32 * sizeof(double);
-}
-
-template <int NR>
 static int near_multi_launch(pb_ctx* c, const float2* dens, double* ys, double eps, int nvalid)
 {
     const PbLevel& lv = c->lev[c->L];
     PB_CUDA(c, cudaFuncSetAttribute(k_near32m<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)near32m_smem<NR>()));
-    k_near32m<NR><<<(c->near_mitems * 32 + 255) / 256, 256, near32m_smem<NR>(), c->st>>>(
+                                    (int)NearM<NR>::smem));
+    k_near32m<NR><<<(c->near_mitems * 32 + 255) / 256, 256, NearM<NR>::smem, c->st>>>(
         c->nt, c->near_mitems, c->near_mitem, c->near_mtiles, c->chunk_leaf, c->chunk_first, lv.begin, c->e32p,
         c->e32n, c->e32l, dens, eps, c->prm.kappa, ys, nvalid);
     PB_LAUNCH(c);
@@ -1020,7 +1048,8 @@ static int near_multi_items(pb_ctx* c)
     if (!c->near_mitem || !c->near_mtiles) return pb_fail(c, PB_ERR_NOMEM, "near setup: out of memory");
     PB_CUDA(c, cudaMemcpyAsync(c->near_mitem, im.data(), sizeof(int4) * im.size(), cudaMemcpyHostToDevice, c->st));
     PB_CUDA(c, cudaMemcpyAsync(c->near_mtiles, tm.data(), sizeof(int) * tm.size(), cudaMemcpyHostToDevice, c->st));
-    return PB_OK;
+    return near_flags(c, c->nchunks, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p, c->near_mitems, c->near_mitem,
+                      c->near_mtiles);
 }
 
 // density buffer of the multi-vector near field and its work items (build lifetime, grown on
