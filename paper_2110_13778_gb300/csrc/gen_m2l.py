@@ -11,11 +11,11 @@ values are used, and reads the scaled moments from shared memory (Ms[b * 33]) fo
 (volatile: kept in registers across FMAs they spilled the accumulators).
 
 M2LWarp<P, W> is the register-blocked two-warp variant used by the FP32 kernel: warp W
-accumulates half of the local coefficients (equal FMA counts), the moments of a block of
-MBLOCK multi-indices sit in registers, and each D^gamma is loaded once per block instead of
-once per FMA, so the shared-memory loads per slot and kernel fall from 3168 to about 740
-(both warps together) at P = 8, with about 170 registers per thread and no spills. Their
-moments are read at Ms[b * 33] (rows padded to 33 words).
+accumulates half of the local coefficients (equal FMA counts) and the moments of a block of
+MBLOCK multi-indices sit in registers. Derivatives and moments come four at a time (16-byte
+shared-memory loads): four consecutive gammas of a slot lie together (Dl[gamma / 4 * 32], a float4
+per lane), and a lane's moments are a row of its own (Ms[b / 4]). 168 loads for 3003 FMAs at P = 8,
+both warps together, about 170 registers per thread and no spills.
 
 Run: python gen_m2l.py > m2l_unrolled.cuh  (the output is committed beside this script).
 """
@@ -29,9 +29,9 @@ GROUP = 4
 # warps with equal FMA counts, and each warp holds the moments of MBLOCK multi-indices at a
 # time in registers
 NWARP = 2
-MBLOCK = {4: 35, 6: 84, 8: 84}
-# row stride of the moments in shared memory for the two-warp bodies: 33, so that the kernel
-# can write one source's moments (lanes over b) without bank conflicts
+MBLOCK = {4: 36, 6: 84, 8: 84}  # multiples of 4
+# row stride of the moments in shared memory of the FP64 kernel: 33, so that it can write one
+# source's moments (lanes over b) without bank conflicts
 MSTRIDE = 33
 
 
@@ -83,6 +83,12 @@ def warp_sets(P, nwarp=NWARP):
     return [sorted(x) for x in sets]
 
 
+def quad(src, names):
+    """One 16-byte load into the named variables (None: not needed)."""
+    out = [f"        v = {src};"]
+    return out + [f"        {n} = v.{c};" for n, c in zip(names, "xyzw") if n]
+
+
 def body_blocked(P, mb, aset):
     """Register-blocked form for the local coefficients a in `aset` (held as L[k], k the
     position in aset): the moments M^b of one block of mb multi-indices are loaded into
@@ -107,15 +113,16 @@ def body_blocked(P, mb, aset):
                     used.add(k)
             if prs:
                 work.append((g, prs))
-        for k in sorted(used):
-            out.append(f"        m{k} = Ms[{blk[k] * MSTRIDE}];")
-        for s in range(0, len(work), GROUP):
-            grp = work[s:s + GROUP]
-            for k, (g, _) in enumerate(grp):
-                out.append(f"        d{k} = Dl[{g * 32}];")
-            for k, (_, prs) in enumerate(grp):
+        for k in sorted({k // 4 for k in used}):  # (blk[0] is a multiple of 4)
+            names = [f"m{4 * k + j}" if 4 * k + j in used else None for j in range(4)]
+            out += quad(f"Ms[{blk[0] // 4 + k}]", names)
+        for g4 in sorted({g // 4 for g, _ in work}):
+            grp = [(g, prs) for g, prs in work if g // 4 == g4]
+            live = {g % 4 for g, _ in grp}
+            out += quad(f"Dl[{g4 * 32}]", [f"d{j}" if j in live else None for j in range(4)])
+            for g, prs in grp:
                 for ia, km in prs:
-                    out.append(f"        L[{ia}] += d{k} * m{km};")
+                    out.append(f"        L[{ia}] += d{g % 4} * m{km};")
     return out
 
 
@@ -156,6 +163,8 @@ def main():
     for P in ORDERS:
         mb = MBLOCK[P]
         for w, aset in enumerate(warp_sets(P)):
+            text = body_blocked(P, mb, aset)
+            ms = {ln.split()[0] for ln in text if ln.split()[0][0] == "m"}
             lines += [
                 "template <>",
                 f"struct M2LWarp<{P}, {w}> {{",
@@ -166,13 +175,14 @@ def main():
                 f"        constexpr short a[{len(aset)}] = {{{', '.join(str(x) for x in aset)}}};",
                 "        return a[k];",
                 "    }",
-                "    template <class R>",
-                "    static __device__ __forceinline__ void run(const R* __restrict__ Dl, const R* __restrict__ Ms, R* L)",
+                "    static __device__ __forceinline__ void run(const float4* __restrict__ Dl, const float4* __restrict__ Ms,",
+                "                                               float* L)",
                 "    {",
-                "        R " + ", ".join(f"m{i}" for i in range(mb)) + ";",
-                "        R " + ", ".join(f"d{i}" for i in range(GROUP)) + ";",
+                "        float4 v;",
+                "        float " + ", ".join(sorted(ms, key=lambda m: int(m[1:]))) + ";",
+                "        float " + ", ".join(f"d{i}" for i in range(GROUP)) + ";",
             ]
-            lines += body_blocked(P, mb, aset)
+            lines += text
             lines += ["    }", "};", ""]
     print("\n".join(lines))
 
