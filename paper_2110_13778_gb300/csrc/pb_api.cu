@@ -63,6 +63,9 @@ static void pb_free_build(pb_ctx* c)
     pb_dg_drop(c);
     c->tc_part = nullptr;
     c->tc_nw = 0;
+    c->tc_list = nullptr;
+    c->tc_cnt = nullptr;
+    c->tc_lpart = nullptr;
     c->bE = nullptr;
     c->bE_n = 0;
     c->q2 = 1;

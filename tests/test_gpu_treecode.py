@@ -116,3 +116,23 @@ def test_molecule_treecode_near_direct():
             assert abs(E - Ed) < 2e-5 * abs(Ed)
         finally:
             pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec,tol", [(pb.PB_FP64, 1e-12), (pb.PB_MIXED, 1e-6)])
+@pytest.mark.parametrize("nc,theta", [(1, 1e-6), (37, 1e-6), (1, 0.03), (33, 0.03)])
+def test_lists_too_short_for_a_small_theta(prec, tol, nc, theta):
+    # about 640 leaves and 128 list places per charge: every leaf (theta 1e-6) or most of them
+    # (0.03) summed directly does not fit, and the call takes the kernel without lists; bars as
+    # for the direct sum above
+    V, T = inputs.icosphere(4, 6.0)
+    qp, q = inputs.ball_charges(nc, 4.5, 9)
+    m = inputs.Mesh(V, T, qp, q)
+    x = inputs.random_density(m.nt, 12)
+    ctx = _ctx(m, prec, 4, leaf=8)
+    try:
+        E = pb.pb_solvation_energy_treecode(ctx, _dev(x), theta)
+        Ed = pb.pb_solvation_energy(ctx, _dev(x))
+        scale = np.abs(q).sum() * np.abs(x).max() * 100.0
+        assert abs(E - Ed) < tol * max(abs(Ed), scale)
+    finally:
+        pb.pb_destroy(ctx)
