@@ -502,6 +502,10 @@ extern "C" int pb_precond_apply(pb_ctx* c, const double* r, double* z)
     PB_ALIVE(c);
     if (!c->built) return pb_fail(c, PB_ERR_STATE, "precond before build_tree");
     if (!r || !z || r == z) return pb_fail(c, PB_ERR_ARG, "precond: bad arguments");
+    if (pb_precond_apply_element(c, r, z)) {
+        PB_CUDA(c, cudaGetLastError());
+        return PB_OK;
+    }
     int rc;
     if ((rc = pb_gather(c, r, c->xs))) return rc;
     if ((rc = pb_precond_apply_sorted(c, c->xs, c->ys))) return rc;

@@ -302,6 +302,7 @@ int pb_far_reserve(pb_ctx* c, int nr);
 int pb_precond_plan(pb_ctx* c);    // precond.cu: block partition (host, synchronises)
 int pb_precond_factor(pb_ctx* c);                                   // precond.cu
 int pb_precond_apply_sorted(pb_ctx* c, const double* r, double* z);
+bool pb_precond_apply_element(pb_ctx* c, const double* r, double* z);  // element order; false: not this form
 int pb_precond_apply_multi(pb_ctx* c, const double* r, long long rstr, double* z, long long zstr, int nr);
 int pb_matvec_sorted_multi(pb_ctx* c, const double* xs, double* ys, int nr);  // pb_api.cu
 int pb_matvec_reserve(pb_ctx* c, int nr);  // pb_api.cu: every buffer a product of nr vectors needs

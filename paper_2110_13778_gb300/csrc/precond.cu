@@ -298,62 +298,90 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_blk_gj_w(const int* __restric
         }
 }
 
-// z = M^-1 r per leaf: the block's slice of r staged once in shared memory (in the working
-// precision), then one warp per row (FP32: two rows) with lanes striding the columns
-template <class R>
-__global__ void k_blk_apply(int nt, const int* __restrict__ begin, const long long* __restrict__ moff,
-                            const R* __restrict__ minv, const double* __restrict__ r, double* __restrict__ z,
-                            long long rstr, long long zstr)
+// z = M^-1 r per block: the block's slice of r staged once in shared memory (in the working precision),
+// then one warp per row with lanes striding the columns. order: r and z in element order (tree
+// position k at order[k]), or nullptr for tree order.
+__device__ __forceinline__ int blk_at(const int* __restrict__ order, int nt, int b, int n, int j)
 {
-    __shared__ __align__(16) R rv[2 * PB_PC_BMAX];
-    r += blockIdx.y * rstr;  // right-hand side blockIdx.y
-    z += blockIdx.y * zstr;
+    const int k = b + (j < n ? j : j - n), e = order ? order[k] : k;
+    return j < n ? e : nt + e;
+}
+
+// FP64
+__global__ void k_blk_apply(int nt, const int* __restrict__ begin, const long long* __restrict__ moff,
+                            const double* __restrict__ minv, const int* __restrict__ order,
+                            const double* __restrict__ r, double* __restrict__ z)
+{
+    __shared__ __align__(16) double rv[2 * PB_PC_BMAX];
     const int c = blockIdx.x;
     const int b = begin[c], n = begin[c + 1] - begin[c], m = 2 * n;
-    const R* Mc = minv + moff[c];
-    for (int j = threadIdx.x; j < m; j += blockDim.x) rv[j] = (R)(j < n ? r[b + j] : r[nt + b + j - n]);
+    const double* Mc = minv + moff[c];
+    for (int j = threadIdx.x; j < m; j += blockDim.x) rv[j] = r[blk_at(order, nt, b, n, j)];
     __syncthreads();
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31, nw = blockDim.x / 32;
-    if constexpr (sizeof(R) == sizeof(float)) {
-        // m is even and every block starts at a multiple of 4 entries (the orders m^2 of the
-        // blocks before it are multiples of 4): rows and the staged slice read in pairs; two rows
-        // per warp at a time, so that twice the loads are in flight
-        const float2* rv2 = reinterpret_cast<const float2*>(rv);
-        for (int i = warp; i < m; i += 2 * nw) {
-            const int i2 = i + nw;
-            const bool two = i2 < m;
-            const float2* row = reinterpret_cast<const float2*>(Mc + (size_t)i * m);
-            const float2* row2 = reinterpret_cast<const float2*>(Mc + (size_t)(two ? i2 : i) * m);
-            float s = 0.f, s2 = 0.f;
-            for (int j = lane; j < m / 2; j += 32) {
-                const float2 a = row[j], a2 = row2[j], v = rv2[j];
-                s += a.x * v.x + a.y * v.y;
-                s2 += a2.x * v.x + a2.y * v.y;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                s += __shfl_xor_sync(0xffffffffu, s, o);
-                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-            }
-            if (lane == 0) {
-                if (i < n) z[b + i] = (double)s;
-                else z[nt + b + i - n] = (double)s;
-                if (two) {
-                    if (i2 < n) z[b + i2] = (double)s2;
-                    else z[nt + b + i2 - n] = (double)s2;
-                }
-            }
-        }
-        return;
-    }
     for (int i = warp; i < m; i += nw) {
-        R s = 0;
+        double s = 0;
         for (int j = lane; j < m; j += 32) s += Mc[(size_t)i * m + j] * rv[j];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            if (i < n) z[b + i] = (double)s;
-            else z[nt + b + i - n] = (double)s;
-        }
+        if (lane == 0) z[blk_at(order, nt, b, n, i)] = s;
     }
+}
+
+// FP32. m is even and every block starts at a multiple of 4 entries (the orders m^2 of the blocks before
+// it are multiples of 4): rows and the staged slice are read in pairs. Four rows per warp at a time, all
+// their loads (up to 12 per lane) issued before the first sum; the four butterflies over the lanes
+// share their steps (each step hands half of the rows over, so that 6 shuffles do what 20 did; the same
+// additions). The results are converted to FP64 32 at a time after the rows: one conversion per row,
+// by one lane each, kept the FP64 pipe 44 % busy. Bound: the blocks from HBM. 327,680 elements (6147
+// blocks, 331 MB): 88.7 us with two rows at a time (3.7 TB/s), 68.4 us now (4.8 TB/s), and no
+// launches that reorder the vectors.
+__global__ void __launch_bounds__(256) k_blk_apply_f(int nt, const int* __restrict__ begin,
+                                                     const long long* __restrict__ moff,
+                                                     const float* __restrict__ minv, const int* __restrict__ order,
+                                                     const double* __restrict__ r, double* __restrict__ z)
+{
+    constexpr int U = (PB_PC_BMAX + 31) / 32;  // pairs of columns per lane
+    __shared__ __align__(16) float rv[2 * PB_PC_BMAX], zv[2 * PB_PC_BMAX];
+    const int c = blockIdx.x;
+    const int b = begin[c], n = begin[c + 1] - begin[c], m = 2 * n;
+    const float* Mc = minv + moff[c];
+    for (int j = threadIdx.x; j < m; j += 256) rv[j] = (float)r[blk_at(order, nt, b, n, j)];
+    __syncthreads();
+    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+    float2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        v[u] = lane + 32 * u < n ? reinterpret_cast<const float2*>(rv)[lane + 32 * u] : make_float2(0.f, 0.f);
+    for (int i = 4 * warp; i < m; i += 32) {
+        float2 a[4][U];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2* row = reinterpret_cast<const float2*>(Mc + (size_t)min(i + q, m - 1) * m);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lane + 32 * u < n) a[q][u] = row[lane + 32 * u];
+        }
+        float s[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s[q] = 0.f;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lane + 32 * u < n) s[q] += a[q][u].x * v[u].x + a[q][u].y * v[u].y;
+        }
+        // lanes < 16 go on with rows 0 and 1, the others with 2 and 3; then one row per 8 lanes
+        const bool hi = lane & 16, hi2 = lane & 8;
+        float t0 = hi ? s[2] : s[0], t1 = hi ? s[3] : s[1];
+        t0 += __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+        t1 += __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+        float t = hi2 ? t1 : t0;
+        t += __shfl_xor_sync(0xffffffffu, hi2 ? t0 : t1, 8);
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        const int row = i + (lane >> 3);  // lane / 8: rows 0, 1, 2, 3
+        if ((lane & 7) == 0 && row < m) zv[row] = t;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < m; j += 256) z[blk_at(order, nt, b, n, j)] = (double)zv[j];
 }
 
 // The same for up to 16 right-hand sides at once (q0 = 16 blockIdx.y, nq of them): each block
@@ -570,15 +598,15 @@ int pb_precond_apply_multi(pb_ctx* c, const double* r, long long rstr, double* z
         const dim3 gm(c->npcblk, (nr + 15) / 16);
         if (c->prm.precision == PB_MIXED) {
             if (nr == 1)
-                k_blk_apply<float><<<c->npcblk, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off, (const float*)c->minv,
-                                                                 r, z, rstr, zstr);
+                k_blk_apply_f<<<c->npcblk, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off, (const float*)c->minv, nullptr, r,
+                                                            z);
             else
                 k_blk_apply_m<float><<<gm, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off, (const float*)c->minv, r,
                                                             z, rstr, zstr, nr);
         } else {
             if (nr == 1)
-                k_blk_apply<double><<<c->npcblk, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off,
-                                                                  (const double*)c->minv, r, z, rstr, zstr);
+                k_blk_apply<<<c->npcblk, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off, (const double*)c->minv, nullptr, r,
+                                                          z);
             else
                 k_blk_apply_m<double><<<gm, 256, 0, c->st>>>(nt, c->pc_begin, c->blk_off,
                                                              (const double*)c->minv, r, z, rstr, zstr, nr);
@@ -595,6 +623,20 @@ int pb_precond_apply_multi(pb_ctx* c, const double* r, long long rstr, double* z
     PB_LAUNCH(c);
     pb_toc(c, PB_T_PRECOND);
     return PB_OK;
+}
+
+// one vector in element order; false where that takes a reordered copy (the caller's)
+bool pb_precond_apply_element(pb_ctx* c, const double* r, double* z)
+{
+    if (c->prm.basis == PB_BASIS_LINEAR || c->prm.precond != PB_PRECOND_BLOCK) return false;
+    pb_tic(c, PB_T_PRECOND);
+    if (c->prm.precision == PB_MIXED)
+        k_blk_apply_f<<<c->npcblk, 256, 0, c->st>>>(c->nt, c->pc_begin, c->blk_off, (const float*)c->minv, c->order, r, z);
+    else
+        k_blk_apply<<<c->npcblk, 256, 0, c->st>>>(c->nt, c->pc_begin, c->blk_off, (const double*)c->minv, c->order, r, z);
+    ++c->nlaunch;
+    pb_toc(c, PB_T_PRECOND);
+    return true;
 }
 
 int pb_precond_apply_sorted(pb_ctx* c, const double* r, double* z)
