@@ -504,11 +504,11 @@ __device__ __forceinline__ void ff_parts(ff r2, ff nxd, ff nyd, ff nxny, ff kap,
     P[5] = ff_mul(P[4], e1);
 }
 
-// The parts of ff_parts, weighted by a quadrature weight w that carries the 1 / (4 pi), added
-// into acc[0 .. PARTS): w is folded into 1 / r once (w / r, w / r^3), so each part costs one
-// product fewer than forming it and then weighting it.
+// The parts of ff_parts, weighted by a quadrature weight w that carries the 1 / (4 pi): the terms
+// X[0 .. PARTS) of the integrals' sums. w is folded into 1 / r once (w / r, w / r^3), so each part costs
+// one product fewer than forming it and then weighting it.
 template <int PARTS>
-__device__ __forceinline__ void ff_parts_w(ff w, ff r2, ff nxd, ff nyd, ff nxny, ff kap, ff* acc)
+__device__ __forceinline__ void ff_parts_w(ff w, ff r2, ff nxd, ff nyd, ff nxny, ff kap, ff* X)
 {
     ff rinv = ff_rsqrt(r2);
     ff r = ff_mul(r2, rinv);
@@ -520,20 +520,20 @@ __device__ __forceinline__ void ff_parts_w(ff w, ff r2, ff nxd, ff nyd, ff nxny,
     ff rinv2 = ff_sqr(rinv);
     const ff wri = ff_mul(w, rinv);       // w / (4 pi r)
     const ff wri3 = ff_mul(wri, rinv2);   // w / (4 pi r^3)
-    acc[0] = ff_sub(acc[0], ff_mul(E, wri));
+    X[0] = ff_neg(ff_mul(E, wri));
     if (PARTS == 2) {
-        acc[1] = ff_sub(acc[1], ff_mul(wri3, ff_mul(c1, nxny)));
+        X[1] = ff_neg(ff_mul(wri3, ff_mul(c1, nxny)));
         return;
     }
     // c3 = -3 g - t^2 - t E (3 + t)
     ff c3 = ff_neg(ff_add(ff_add(ff_mul_f(g, 3.0f), ff_sqr(t)), ff_mul(tE, ff_add_f(t, 3.0f))));
-    acc[1] = ff_add(acc[1], ff_mul(wri3, ff_sub(ff_mul(ff_mul(c3, ff_mul(nxd, nyd)), rinv2), ff_mul(c1, nxny))));
+    X[1] = ff_mul(wri3, ff_sub(ff_mul(ff_mul(c3, ff_mul(nxd, nyd)), rinv2), ff_mul(c1, nxny)));
     ff e1 = ff_add_f(ff_neg(c1), 1.0f);
     const ff p2 = ff_mul(nyd, wri3), p4 = ff_mul(nxd, wri3);
-    acc[2] = ff_add(acc[2], p2);
-    acc[3] = ff_add(acc[3], ff_mul(p2, e1));
-    acc[4] = ff_add(acc[4], p4);
-    acc[5] = ff_add(acc[5], ff_mul(p4, e1));
+    X[2] = p2;
+    X[3] = ff_mul(p2, e1);
+    X[4] = p4;
+    X[5] = ff_mul(p4, e1);
 }
 
 __device__ __forceinline__ ff ff_dot3(const ff* a, const ff* b)
@@ -647,23 +647,27 @@ static void ss_table(int qs, SsTable& T)
         }
 }
 
-// The cube points of one pair's class (lane, lane + stride, ...), one body per class: CLS = 0,
-// a shared vertex (all four coefficients); 1, a shared edge (b0 = 0: eQ0 = eP0 is merged into
-// a0); 2, identical triangles, where x - y lies in the triangle's own plane (only a0, a1 are
-// nonzero) and both normal projections vanish, so only parts 0 and 1 of the kernel remain.
-// Pairs are grouped by class, so the warps that run each body are uniform.
-template <int CLS>
-__device__ __forceinline__ void ss_points_ff(int lane, const float2* __restrict__ tab, int tn, int off, int cnt,
-                                             const ff (*eP)[3], const ff (*eQ)[3], const ff* proj, ff nxny, ff kap,
-                                             ff* acc, int stride)
+// The cube points of one pair's class, one body per class: CLS = 0, a shared vertex (all four
+// coefficients); 1, a shared edge (b0 = 0: eQ0 = eP0 is merged into a0); 2, identical triangles, where
+// x - y lies in the triangle's own plane (only a0, a1 are nonzero) and both normal projections vanish, so
+// only parts 0 and 1 of the kernel remain. Pairs are grouped by class, so the warps that run each
+// body are uniform. LPP lanes share a pair: each takes one of LPP consecutive points, and lane m then
+// adds part m of the points in their order (the terms travel by shuffles among the lanes of gmask), so that
+// every sum is made in the order, and with the bits, of one lane alone.
+template <int CLS, int LPP>
+__device__ __forceinline__ void ss_points_ff(int sub, unsigned gmask, const float2* __restrict__ tab, int tn, int off,
+                                             int cnt, const ff (*eP)[3], const ff (*eQ)[3], const ff* proj, ff nxny, ff kap,
+                                             ff* acc)
 {
-    for (int i = off + lane; i < off + cnt; i += stride) {
+    constexpr int PARTS = CLS == 2 ? 2 : 6;
+    for (int i0 = off; i0 < off + cnt; i0 += LPP) {
+        const int i = LPP == 1 ? i0 : min(i0 + sub, off + cnt - 1);
         const ff a0 = ld_ff(tab + i), a1 = ld_ff(tab + tn + i), w = ld_ff(tab + 4 * tn + i);
-        ff d[3];
+        ff d[3], X[6];
         if (CLS == 2) {
             for (int c = 0; c < 3; ++c) d[c] = ff_add(ff_mul(a0, eP[0][c]), ff_mul(a1, eP[1][c]));
             const ff r2 = ff_add(ff_add(ff_sqr(d[0]), ff_sqr(d[1])), ff_sqr(d[2]));
-            ff_parts_w<2>(w, r2, ff{0.f, 0.f}, ff{0.f, 0.f}, nxny, kap, acc);
+            ff_parts_w<2>(w, r2, ff{0.f, 0.f}, ff{0.f, 0.f}, nxny, kap, X);
         } else {
             const ff b0 = CLS == 1 ? ff{0.f, 0.f} : ld_ff(tab + 2 * tn + i), b1 = ld_ff(tab + 3 * tn + i);
             for (int c = 0; c < 3; ++c) {
@@ -675,8 +679,28 @@ __device__ __forceinline__ void ss_points_ff(int lane, const float2* __restrict_
             // proj = {n_x.eQ0, n_x.eQ1, n_y.eP0, n_y.eP1}
             const ff nxd = ff_neg(CLS == 1 ? ff_mul(b1, proj[1]) : ff_add(ff_mul(b0, proj[0]), ff_mul(b1, proj[1])));
             const ff nyd = ff_add(ff_mul(a0, proj[2]), ff_mul(a1, proj[3]));
-            ff_parts_w<6>(w, r2, nxd, nyd, nxny, kap, acc);
+            ff_parts_w<6>(w, r2, nxd, nyd, nxny, kap, X);
         }
+        if (LPP == 1) {
+#pragma unroll
+            for (int m = 0; m < PARTS; ++m) acc[m] = ff_add(acc[m], X[m]);
+        } else {
+            const int n = min(LPP, off + cnt - i0);
+            for (int q = 0; q < n; ++q) {
+                ff x = {0.f, 0.f};
+#pragma unroll
+                for (int m = 0; m < PARTS; ++m) {
+                    const float h = __shfl_sync(gmask, X[m].h, q, LPP), l = __shfl_sync(gmask, X[m].l, q, LPP);
+                    if (sub == m) x = {h, l};
+                }
+                acc[0] = ff_add(acc[0], x);  // (lane m: part m)
+            }
+        }
+    }
+    if (LPP > 1) {
+        const ff mine = acc[0];
+#pragma unroll
+        for (int m = 0; m < PARTS; ++m) acc[m] = {__shfl_sync(gmask, mine.h, m, LPP), __shfl_sync(gmask, mine.l, m, LPP)};
     }
 }
 
@@ -719,15 +743,16 @@ __global__ void k_canon(int nt, const int* __restrict__ toff, const int* __restr
         for (int g = 0; g < 3; ++g) cnt[g * nt + k] = n[g];
 }
 
-// SS_LPP threads per unordered touching pair (1: one thread per pair). Pairs are grouped by
-// class, so the pairs of a warp share one trip count and read the same (or neighbouring) table
-// entries together. With one thread per pair no per-pair work is repeated across lanes, no
-// cross-lane reduction is needed and no lane idles in a last, partial round of points (the
-// warp-per-pair form of this kernel left 10 % of its point slots idle and repeated the pair's
-// setup on 32 lanes). Both ordered entries, (k, j) and (j, k), come from the same sums and the
-// same one-point evaluation (under the exchange d -> -d, n_x <-> n_y the parts 0 and 1 are
-// unchanged and parts 2..5 map to -4, -5, -2, -3).
-#define SS_LPP 1
+// LPP threads per unordered touching pair. Pairs are grouped by class, so the pairs of a warp share one
+// trip count and read the same (or neighbouring) table entries together. One thread per pair repeats no
+// work across lanes, needs no cross-lane step and leaves no lane idle in a last, partial round of points (a
+// warp per pair left 10 % of its point slots idle and repeated the pair's setup on 32 lanes): the choice
+// where the pairs fill the GPU. Below that a thread's hundreds of points are the launch's length: eight
+// lanes per pair there (8930 pairs: 272 -> 98 us; 57,000 pairs: 365 us, with eight lanes 406; the line lies
+// at 36,000, where the eight lanes' time, 7 us per 1000 pairs, reaches the length of one thread). Both ordered entries, (k, j) and (j, k), come from
+// the same sums and the same one-point evaluation (under the exchange d -> -d, n_x <-> n_y the parts 0
+// and 1 are unchanged and parts 2..5 map to -4, -5, -2, -3).
+template <int LPP>
 __global__ void __launch_bounds__(128) k_singular_ff1(int ncanon, const int* __restrict__ ncanon_dev,
                                                       const int* __restrict__ ck, const int* __restrict__ cp,
                                                       const int* __restrict__ toff, const int* __restrict__ tj,
@@ -736,8 +761,8 @@ __global__ void __launch_bounds__(128) k_singular_ff1(int ncanon, const int* __r
                                                       ff kap, ff epsf, ff iepsf, double* __restrict__ corr)
 {
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int w = tid / SS_LPP, sub = tid % SS_LPP;
-    // (all SS_LPP threads of a pair leave together: the shuffles below stay within live groups)
+    const int w = tid / LPP, sub = tid % LPP;
+    // (all LPP threads of a pair leave together: the shuffles below stay within live groups)
     if (w >= ncanon || w >= *ncanon_dev) return;  // allocated pairs, and those the scan found
     const int k = ck[w];
     const long long pair = cp[w];
@@ -787,16 +812,11 @@ __global__ void __launch_bounds__(128) k_singular_ff1(int ncanon, const int* __r
     }
     const int off = ns == 3 ? toffs.z : ns == 2 ? toffs.y : toffs.x;
     const int cnt = ns == 3 ? tcnts.z : ns == 2 ? tcnts.y : tcnts.x;
-    if (ns == 3) ss_points_ff<2>(sub, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc, SS_LPP);
-    else if (ns == 2) ss_points_ff<1>(sub, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc, SS_LPP);
-    else ss_points_ff<0>(sub, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc, SS_LPP);
-    // the pair's own SS_LPP lanes, all alive (a pair's lanes leave together)
-    const unsigned gmask = ((1u << SS_LPP) - 1u) << ((threadIdx.x & 31) & ~(SS_LPP - 1));
-    for (int m = 0; m < 6; ++m)
-        for (int o = 1; o < SS_LPP; o <<= 1) {
-            ff v = {__shfl_xor_sync(gmask, acc[m].h, o), __shfl_xor_sync(gmask, acc[m].l, o)};
-            acc[m] = ff_add(acc[m], v);
-        }
+    // the pair's own lanes, all alive (a pair's lanes leave together)
+    const unsigned gmask = (unsigned)(((1ull << LPP) - 1ull) << ((threadIdx.x & 31) & ~(LPP - 1)));
+    if (ns == 3) ss_points_ff<2, LPP>(sub, gmask, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc);
+    else if (ns == 2) ss_points_ff<1, LPP>(sub, gmask, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc);
+    else ss_points_ff<0, LPP>(sub, gmask, tab, tn, off, cnt, eP, eQ, proj, nxny, kap, acc);
     if (sub > 1) return;
     const ff Ak = ld_ff(rk + 15), Aj = ld_ff(rj + 15);
     const ff AA = ff_mul(Ak, Aj);
@@ -829,7 +849,7 @@ __global__ void __launch_bounds__(128) k_singular_ff1(int ncanon, const int* __r
         o0[0] = make_double2(ff_to(I[0][0]), ff_to(I[0][1]));
         o0[1] = make_double2(ff_to(I[0][2]), ff_to(I[0][3]));
     }
-    if (sub == (SS_LPP > 1 ? 1 : 0) && k != j && qr < toff[j + 1]) {
+    if (sub == (LPP > 1 ? 1 : 0) && k != j && qr < toff[j + 1]) {
         double2* o1 = (double2*)(corr + 4 * qr);
         o1[0] = make_double2(ff_to(I[1][0]), ff_to(I[1][1]));
         o1[1] = make_double2(ff_to(I[1][2]), ff_to(I[1][3]));
@@ -936,10 +956,12 @@ int pb_touching_and_singular(pb_ctx* c)
     k_canon<1><<<nblk(nt, B), B, 0, c->st>>>(nt, c->touch_off, c->touch_j, c->order, c->stris, nullptr, coff, ck, cp,
                                              ncanon);
     PB_LAUNCH(c);
-    k_singular_ff1<<<nblk((long long)ncanon * SS_LPP, 128), 128, 0, c->st>>>(ncanon, coff + 3 * nt, ck, cp, c->touch_off, c->touch_j, c->stris, erec, tab,
-                                                    T.n, make_int3(T.off[0], T.off[1], T.off[2]),
-                                                    make_int3(T.cnt[0], T.cnt[1], T.cnt[2]), ff_from(c->prm.kappa),
-                                                    ff_from(eps), ff_from(1.0 / eps), c->corr);
+    const bool few = ncanon < 36000;
+    auto* kern = few ? k_singular_ff1<8> : k_singular_ff1<1>;
+    kern<<<nblk((long long)ncanon * (few ? 8 : 1), 128), 128, 0, c->st>>>(
+        ncanon, coff + 3 * nt, ck, cp, c->touch_off, c->touch_j, c->stris, erec, tab, T.n,
+        make_int3(T.off[0], T.off[1], T.off[2]), make_int3(T.cnt[0], T.cnt[1], T.cnt[2]), ff_from(c->prm.kappa),
+        ff_from(eps), ff_from(1.0 / eps), c->corr);
     PB_LAUNCH(c);
     // (the singular pass is left running)
     return PB_OK;
