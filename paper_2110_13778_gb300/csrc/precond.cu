@@ -262,15 +262,26 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_blk_gj_w(const int* __restric
             const float ia = 1.f / piv;
             const int pa = p >> 5, pl = p & 31;
             if (lane == pl) used |= 1u << pa;
-            // row p of this warp's columns, from the lane that holds it
+            // row p of this warp's columns, from the lane that holds it: with six rows per lane by one
+            // uniform branch on p / 32 (class of order <= 192: 2266 -> 2074 us on 327,680 elements), with
+            // fewer by selections (order <= 128: 1363 us, 1511 by the branch)
             float rk[MB];
+            if constexpr (MA > 4) {
 #pragma unroll
-            for (int b = 0; b < MB; ++b) {
-                float x = v[0][b];
+                for (int a = 0; a < MA; ++a)
+                    if (a == pa) {
 #pragma unroll
-                for (int a = 1; a < MA; ++a)
-                    if (a == pa) x = v[a][b];
-                rk[b] = __shfl_sync(0xffffffffu, x, pl) * ia;
+                        for (int b = 0; b < MB; ++b) rk[b] = __shfl_sync(0xffffffffu, v[a][b], pl) * ia;
+                    }
+            } else {
+#pragma unroll
+                for (int b = 0; b < MB; ++b) {
+                    float x = v[0][b];
+#pragma unroll
+                    for (int a = 1; a < MA; ++a)
+                        if (a == pa) x = v[a][b];
+                    rk[b] = __shfl_sync(0xffffffffu, x, pl) * ia;
+                }
             }
             const bool ownk = warp == kw;
 #pragma unroll

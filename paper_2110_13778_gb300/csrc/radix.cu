@@ -1,8 +1,9 @@
 // Prefix sums and the Morton-key radix sort of the tree build (Section 2.4, cluster
 // hierarchy: elements ordered by the Morton code of their centroids).
 //
-// Exclusive scan: per-tile sums, a scan of the tile sums in one block, then each tile scans
-// itself and adds its offset. Radix sort: least-significant-digit first, 8-bit digits; each
+// Exclusive scan: per-tile sums, then each tile scans itself and adds the sums of the tiles before it
+// (from SC_ROWS tiles on, a scan of the tile sums in one block comes between); up to SC_ONE values in
+// one block and one launch (a build of 1280 elements makes 11 scans: 126 -> 37 us with four launches each). Radix sort: least-significant-digit first, 8-bit digits; each
 // pass counts the digits of every tile of 256 keys, scans the counts digit-major (digit d of
 // tile t lands after every smaller digit and after digit d of the earlier tiles), and
 // scatters. Within a tile the rank among equal digits keeps the input order (peers found by a
@@ -13,6 +14,8 @@
 #include "pb_internal.cuh"
 
 #define SC_T 1024    // elements per scan tile (256 threads x 4)
+#define SC_ONE 16384 // values of a one-block scan (1024 threads x 16): a launch in place of two to four
+#define SC_ROWS 4096 // tiles whose sums every tile adds up itself
 #define RS_T 256     // keys per radix tile (one per thread)
 #define RS_BINS 256
 
@@ -63,50 +66,93 @@ __global__ void k_scan_sums(int ntile, int* __restrict__ tsum)
     if (threadIdx.x == 0) tsum[ntile] = carry;
 }
 
-__global__ void k_scan_apply(int n, const int* __restrict__ in, const int* __restrict__ tsum, int* __restrict__ out)
+// the block's inclusive scan of one value per thread (blockDim.x <= 1024); *total: the block's sum
+__device__ __forceinline__ int block_scan(int v, int* wsum, int* total)
 {
-    __shared__ int wsum[8];
-    const int base = blockIdx.x * SC_T + threadIdx.x * 4;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int v[4], s = 0;
-    for (int q = 0; q < 4; ++q) {
-        v[q] = base + q < n ? in[base + q] : 0;
-        s += v[q];
-    }
-    int inc = s;  // inclusive scan of the thread sums within the warp
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int inc = v;
     for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
     if (lane == 31) wsum[w] = inc;
     __syncthreads();
-    int woff = 0;
-    for (int k = 0; k < w; ++k) woff += wsum[k];
-    int run = tsum[blockIdx.x] + woff + inc - s;
+    if (w == 0) {
+        int x = lane < nw ? wsum[lane] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += t;
+        }
+        if (lane < nw) wsum[lane] = x;
+    }
+    __syncthreads();
+    *total = wsum[nw - 1];
+    return inc + (w ? wsum[w - 1] : 0);
+}
+
+// scanned: tsum holds the exclusive scan of the tile sums, else the tile sums
+__global__ void k_scan_apply(int n, const int* __restrict__ in, const int* __restrict__ tsum, int scanned,
+                             int* __restrict__ out)
+{
+    __shared__ int wsum[32], wsum2[32];
+    const int base = blockIdx.x * SC_T + threadIdx.x * 4;
+    int before = 0;
+    if (scanned) {
+        before = tsum[blockIdx.x];
+    } else {
+        int s = 0;
+        for (int i = threadIdx.x; i < blockIdx.x; i += 256) s += tsum[i];
+        block_scan(s, wsum2, &before);
+    }
+    int v[4], s = 0, total;
+    for (int q = 0; q < 4; ++q) {
+        v[q] = base + q < n ? in[base + q] : 0;
+        s += v[q];
+    }
+    int run = before + block_scan(s, wsum, &total) - s;
     for (int q = 0; q < 4; ++q) {
         if (base + q < n) out[base + q] = run;
         run += v[q];
     }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + total;
 }
 
-__global__ void k_scan_total(int n, const int* __restrict__ tsum, int ntile, int* __restrict__ out)
+__global__ void __launch_bounds__(1024) k_scan_one(int n, const int* __restrict__ in, int* __restrict__ out)
 {
-    out[n] = tsum[ntile];
+    __shared__ int wsum[32];
+    const int per = (n + 1023) / 1024, b = threadIdx.x * per;  // (at most 16)
+    int s = 0, total;
+    for (int q = 0; q < per; ++q)
+        if (b + q < n) s += in[b + q];
+    int run = block_scan(s, wsum, &total) - s;
+    for (int q = 0; q < per; ++q)
+        if (b + q < n) {
+            const int v = in[b + q];
+            out[b + q] = run;
+            run += v;
+        }
+    if (threadIdx.x == 0) out[n] = total;
 }
 
 // out[i] = sum of in[0..i) for i = 0..n (out[n] the total); queued on c->st
 int pb_scan_exclusive(pb_ctx* c, const int* in, int* out, int n)
 {
+    if (n <= SC_ONE) {
+        k_scan_one<<<1, 1024, 0, c->st>>>(n, in, out);
+        PB_LAUNCH(c);
+        return PB_OK;
+    }
     const int ntile = std::max(1, (n + SC_T - 1) / SC_T);
     int* tsum = nullptr;
     PB_CUDA(c, cudaMallocFromPoolAsync((void**)&tsum, sizeof(int) * (ntile + 1), c->pool, c->st));
     k_scan_tiles<<<ntile, 256, 0, c->st>>>(n, in, tsum);
     PB_LAUNCH(c);
-    k_scan_sums<<<1, 1024, 0, c->st>>>(ntile, tsum);
-    PB_LAUNCH(c);
-    k_scan_apply<<<ntile, 256, 0, c->st>>>(n, in, tsum, out);
-    PB_LAUNCH(c);
-    k_scan_total<<<1, 1, 0, c->st>>>(n, tsum, ntile, out);
+    const bool rows = ntile > SC_ROWS;
+    if (rows) {
+        k_scan_sums<<<1, 1024, 0, c->st>>>(ntile, tsum);
+        PB_LAUNCH(c);
+    }
+    k_scan_apply<<<ntile, 256, 0, c->st>>>(n, in, tsum, rows, out);
     PB_LAUNCH(c);
     PB_CUDA(c, cudaFreeAsync(tsum, c->st));
     return PB_OK;

@@ -358,3 +358,28 @@ def test_mixed_near_tiles_against_fp64(kappa, leaf, qr):
         finally:
             pb.pb_destroy(ctx)
     assert _rel(got[1], got[0]) < 6e-7
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 16383, 16384, 16385, 16384 + 1024])
+def test_scans_across_one_block_and_tiles(n):
+    # the build's scans at the edges of the one-block form (16384 values) and of the tiles behind it:
+    # the order, the cluster ranges and the touching counts of a mesh of n triangles
+    V, T = inputs.icosphere(5 if n > 5120 else 4, 3.0)
+    T = T[:n]
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    ctx = _ctx(m, leaf_size=24, eta0=0.8, p=2, precision=pb.PB_MIXED, precond=pb.PB_PRECOND_DIAG)
+    try:
+        st, order, lb, nc, ni, ic, ii = pb.pb_get_tree(ctx, m.nt)
+        tr = fmm.Tree(V, T, leaf_size=24, eta0=0.8)
+        assert np.array_equal(order, tr.order)
+        assert np.array_equal(lb[-len(tr.begin[tr.L]):], tr.begin[tr.L])
+        share = {}
+        for t in T:
+            for v in t:
+                share[v] = share.get(v, 0) + 1
+        # touching ordered pairs: by vertex, minus those counted twice or three times (shared edges, i == j)
+        E = np.sort(T[:, [0, 1, 1, 2, 2, 0]].reshape(-1, 2), 1)
+        _, k = np.unique(E, axis=0, return_counts=True)
+        assert st["touching"] == sum(c * c for c in share.values()) - int((k * k).sum()) + m.nt
+    finally:
+        pb.pb_destroy(ctx)
