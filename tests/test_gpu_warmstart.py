@@ -108,7 +108,9 @@ def test_gradient_matches_oracle(net, n):
 
 
 @pytest.mark.parametrize("shape,n", [((18, 128, 3, 2), 127), ((18, 128, 3, 2), 129), ((18, 128, 3, 2), 4097),
-                                     ((5, 64, 2, 3), 300), ((40, 256, 1, 33), 1000), ((16, 144, 2, 17), 513)])
+                                     ((5, 64, 2, 3), 300), ((40, 256, 1, 33), 1000), ((16, 144, 2, 17), 513),
+                                     ((5, 128, 1, 16), 200), ((32, 128, 2, 3), 640), ((18, 128, 4, 2), 257),
+                                     ((17, 128, 3, 1), 1)])
 def test_gradient_tiles_and_row_slices(shape, n):
     # one row slice and several, with remainders; tiles of 16 to 128 columns and two tiles per
     # matrix; the same bfloat16 rounding points as the oracle's emulation (bar: 2e-2 as above)
