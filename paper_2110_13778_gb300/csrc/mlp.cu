@@ -11,12 +11,14 @@
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <vector>
 
 #include "pb_internal.cuh"
 
 #define MLP_MAXL 8
+#define MLP_STAGE (1 << 20)
 
 struct pb_mlp {
     int nin = 0, width = 0, depth = 0, nout = 0;  // depth = number of hidden layers
@@ -34,8 +36,9 @@ struct pb_mlp {
     __nv_bfloat16* dZb[2] = {};
     float* part = nullptr;
     int part_n = 0;
-    float* lossbuf = nullptr;
-    int* derr = nullptr;  // set by the tensor-core inference when a bounded wait gives up
+    float* lossbuf = nullptr;  // the loss, after the gradient in G
+    int* derr = nullptr;  // after the loss: set when a bounded wait on the tensor cores gives up
+    float* hbuf = nullptr;  // pinned copy of G, the loss and the flag (MLP_STAGE parameters at most, else null)
     long long nparam = 0;
     int adam_t = 0;
     std::string err;
@@ -562,11 +565,16 @@ extern "C" int pb_mlp_create(int nin, int width, int depth, int nout, unsigned l
     bool ok = cudaMalloc(&m->W, sizeof(float) * o) == cudaSuccess;
     ok &= cudaMalloc(&m->Wm, sizeof(float) * o) == cudaSuccess;
     ok &= cudaMalloc(&m->Wv, sizeof(float) * o) == cudaSuccess;
-    ok &= cudaMalloc(&m->G, sizeof(float) * o) == cudaSuccess;
+    ok &= cudaMalloc(&m->G, sizeof(float) * (o + 2)) == cudaSuccess;
     ok &= cudaMalloc(&m->Wb, sizeof(__nv_bfloat16) * o) == cudaSuccess;
-    ok &= cudaMalloc(&m->lossbuf, sizeof(float)) == cudaSuccess;
-    ok &= cudaMalloc(&m->derr, sizeof(int)) == cudaSuccess;
-    ok &= ok && cudaMemset(m->derr, 0, sizeof(int)) == cudaSuccess;
+    m->lossbuf = m->G + o;
+    m->derr = (int*)(m->G + o + 1);
+    ok = ok && cudaMemset(m->derr, 0, sizeof(int)) == cudaSuccess;
+    // (without it, should the host have no pinned memory left, the copies go one by one)
+    if (ok && o <= MLP_STAGE && cudaMallocHost(&m->hbuf, sizeof(float) * (o + 2)) != cudaSuccess) {
+        cudaGetLastError();
+        m->hbuf = nullptr;
+    }
     if (!ok) {
         cudaGetLastError();
         delete m;
@@ -609,8 +617,7 @@ extern "C" int pb_mlp_destroy(pb_mlp* m)
     cudaFree(m->Wv);
     cudaFree(m->G);
     cudaFree(m->Wb);
-    cudaFree(m->lossbuf);
-    cudaFree(m->derr);
+    cudaFreeHost(m->hbuf);
     cudaFree(m->Z);
     for (int l = 0; l <= MLP_MAXL; ++l) cudaFree(m->Ab[l]);
     for (auto& d : m->dZb) cudaFree(d);
@@ -1171,6 +1178,16 @@ extern "C" int pb_mlp_gradient(pb_mlp* m, const float* X, const float* T, int n,
     if (!m || !X || !T || n < 1) return PB_ERR_ARG;
     int rc = mlp_loss_grad(m, X, T, n);
     if (rc) return rc;
+    if (m->hbuf && grad_host) {  // gradient, loss and flag in one copy
+        if (cudaMemcpyAsync(m->hbuf, m->G, sizeof(float) * (m->nparam + 2), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
+            return mlp_fail(m, PB_ERR_CUDA, "mlp: copy failed");
+        if (cudaStreamSynchronize(m->st) != cudaSuccess) return mlp_fail(m, PB_ERR_CUDA, "mlp: sync failed");
+        if (loss) *loss = m->hbuf[m->nparam];
+        memcpy(grad_host, m->hbuf, sizeof(float) * m->nparam);
+        int herr;
+        memcpy(&herr, m->hbuf + m->nparam + 1, sizeof(int));
+        return herr ? mlp_check_err(m) : PB_OK;
+    }
     if (loss && cudaMemcpyAsync(loss, m->lossbuf, sizeof(float), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
         return mlp_fail(m, PB_ERR_CUDA, "mlp: copy failed");
     if (grad_host &&
