@@ -752,8 +752,11 @@ __global__ void k_canon(int nt, const int* __restrict__ toff, const int* __restr
 // at 36,000, where the eight lanes' time, 7 us per 1000 pairs, reaches the length of one thread). Both ordered entries, (k, j) and (j, k), come from
 // the same sums and the same one-point evaluation (under the exchange d -> -d, n_x <-> n_y the parts 0
 // and 1 are unchanged and parts 2..5 map to -4, -5, -2, -3).
+// Bound: FP32 issue, the pipe being held up by register-bank conflicts; the register budget decides
+// how they fall (327,680 elements: 96 registers, the compiler's own choice, 10.95 ms; 128 registers
+// 9.73; 80: 10.07; 64: 10.74).
 template <int LPP>
-__global__ void __launch_bounds__(128) k_singular_ff1(int ncanon, const int* __restrict__ ncanon_dev,
+__global__ void __launch_bounds__(128, 4) k_singular_ff1(int ncanon, const int* __restrict__ ncanon_dev,
                                                       const int* __restrict__ ck, const int* __restrict__ cp,
                                                       const int* __restrict__ toff, const int* __restrict__ tj,
                                                       const int* __restrict__ stris, const float2* __restrict__ erec,
