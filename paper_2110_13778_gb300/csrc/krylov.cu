@@ -101,19 +101,29 @@ __global__ void __launch_bounds__(KB) k_rhs(int nt, int nc, const double4_32a* _
 // two halves of every f32x2 operation, and each staged charge is stored duplicated in both
 // halves (x, x, y, y), (z, z, q, q) and (x_lo, x_lo, y_lo, y_lo), (z_lo, z_lo, 0, 0), so one
 // instruction does the work of both pair evaluations; only the reciprocal square root runs per
-// half.
-__global__ void __launch_bounds__(KB, 4) k_rhs_x2(int nt, int nc, const double4_32a* __restrict__ ep,
-                                               const double4_32a* __restrict__ en, const double* __restrict__ qpos,
-                                               const double* __restrict__ q, double eps1, double* __restrict__ b)
+// half. The block's threads fall into G groups, which take the tiles of KB charges in turn for the
+// same 2 KB / G elements (FP64 sums of the tiles' sums, added up in group order). Bound: the FMA
+// pipe, once there are warps enough: a thread for every two elements and all charges leaves 8 warps on
+// an SM at 81,920 elements (900 charges: 103 us with one group, 75 with four; 118 us with rsqrtf's
+// steps for subnormal arguments, which squared distances of these coordinates never are).
+template <int G>
+__global__ void __launch_bounds__(KB, G > 1 ? 3 : 4) k_rhs_x2(int nt, int nc, const double4_32a* __restrict__ ep,
+                                                              const double4_32a* __restrict__ en,
+                                                              const double* __restrict__ qpos,
+                                                              const double* __restrict__ q, double eps1,
+                                                              double* __restrict__ b)
 {
-    __shared__ float4 sq[4][KB];
-    const int k0 = blockIdx.x * 2 * KB + threadIdx.x;
+    constexpr int GT = KB / G;
+    extern __shared__ float4 rhs_sm[];
+    const int g = threadIdx.x / GT, i = threadIdx.x % GT;
+    const float4* sq = rhs_sm + g * 4 * KB;  // [G][4][KB]: the group's tile
+    const int k0 = blockIdx.x * 2 * GT + i;
     float ph[2][3], pl[2][3], nr[2][3];
     double w[2];
     bool act[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int k = k0 + u * KB;
+        const int k = k0 + u * GT;
         act[u] = k < nt;
         double4_32a p = make_double4_32a(0, 0, 0, 0), n = p;
         if (act[u]) {
@@ -134,31 +144,34 @@ __global__ void __launch_bounds__(KB, 4) k_rhs_x2(int nt, int nc, const double4_
     const f2x nx = x2_pack(nr[0][0], nr[1][0]), ny = x2_pack(nr[0][1], nr[1][1]), nz = x2_pack(nr[0][2], nr[1][2]);
     double s1[2] = {0.0, 0.0}, s2[2] = {0.0, 0.0};
     const double i4pi = 0.07957747154594767;
-    for (int t0 = 0; t0 < nc; t0 += KB) {
+    for (int t0 = 0; t0 < nc; t0 += G * KB) {
         __syncthreads();
-        if (t0 + threadIdx.x < nc) {
-            const int t = t0 + threadIdx.x;
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+            const int t = t0 + h * KB + threadIdx.x;
+            if (t >= nc) break;
+            float4* st = rhs_sm + h * 4 * KB + threadIdx.x;
             const double v[3] = {qpos[3 * t], qpos[3 * t + 1], qpos[3 * t + 2]};
-            const float h[3] = {(float)v[0], (float)v[1], (float)v[2]};
-            const float l[3] = {(float)(v[0] - (double)h[0]), (float)(v[1] - (double)h[1]), (float)(v[2] - (double)h[2])};
+            const float hi[3] = {(float)v[0], (float)v[1], (float)v[2]};
+            const float l[3] = {(float)(v[0] - (double)hi[0]), (float)(v[1] - (double)hi[1]), (float)(v[2] - (double)hi[2])};
             const float qq = (float)q[t];
-            sq[0][threadIdx.x] = make_float4(h[0], h[0], h[1], h[1]);
-            sq[1][threadIdx.x] = make_float4(h[2], h[2], qq, qq);
-            sq[2][threadIdx.x] = make_float4(l[0], l[0], l[1], l[1]);
-            sq[3][threadIdx.x] = make_float4(l[2], l[2], 0.f, 0.f);
+            st[0] = make_float4(hi[0], hi[0], hi[1], hi[1]);
+            st[KB] = make_float4(hi[2], hi[2], qq, qq);
+            st[2 * KB] = make_float4(l[0], l[0], l[1], l[1]);
+            st[3 * KB] = make_float4(l[2], l[2], 0.f, 0.f);
         }
         __syncthreads();
-        const int m = min(KB, nc - t0);
+        const int m = min(KB, nc - (t0 + g * KB));
         f2x a1 = x2_dup(0.f), a2 = x2_dup(0.f);
         for (int t = 0; t < m; ++t) {
-            const float4 g0 = sq[0][t], g1 = sq[1][t], g2 = sq[2][t], g3 = sq[3][t];
+            const float4 g0 = sq[t], g1 = sq[KB + t], g2 = sq[2 * KB + t], g3 = sq[3 * KB + t];
             const f2x dx = x2_add(x2_sub(px, x2_pack(g0.x, g0.y)), x2_sub(lx, x2_pack(g2.x, g2.y)));
             const f2x dy = x2_add(x2_sub(py, x2_pack(g0.z, g0.w)), x2_sub(ly, x2_pack(g2.z, g2.w)));
             const f2x dz = x2_add(x2_sub(pz, x2_pack(g1.x, g1.y)), x2_sub(lz, x2_pack(g3.x, g3.y)));
             const f2x r2 = x2_fma(dz, dz, x2_fma(dy, dy, x2_mul(dx, dx)));
             float ra, rb;
             x2_unpack(r2, ra, rb);
-            const f2x ri = x2_pack(rsqrtf(ra), rsqrtf(rb));
+            const f2x ri = x2_pack(rsqrt_ftz(ra), rsqrt_ftz(rb));
             const f2x nd = x2_fma(nz, dz, x2_fma(ny, dy, x2_mul(nx, dx)));
             const f2x qr = x2_mul(x2_pack(g1.z, g1.w), ri);
             a1 = x2_add(a1, qr);
@@ -172,14 +185,41 @@ __global__ void __launch_bounds__(KB, 4) k_rhs_x2(int nt, int nc, const double4_
         s2[0] += (double)u0;
         s2[1] += (double)u1;
     }
+    if (G > 1) {
+        double* sh = (double*)rhs_sm;  // [G][4][GT]
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            sh[(4 * g + u) * GT + i] = s1[u];
+            sh[(4 * g + 2 + u) * GT + i] = s2[u];
+        }
+        __syncthreads();
+        if (g > 0) return;
+#pragma unroll
+        for (int h = 1; h < G; ++h)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                s1[u] += sh[(4 * h + u) * GT + i];
+                s2[u] += sh[(4 * h + 2 + u) * GT + i];
+            }
+    }
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int k = k0 + u * KB;
+        const int k = k0 + u * GT;
         if (act[u]) {
             b[k] = w[u] * s1[u] * i4pi / eps1;
             b[nt + k] = w[u] * s2[u] * i4pi / eps1;
         }
     }
+}
+template <int G>
+static int rhs_x2(pb_ctx* c, int nt, const double4_32a* ep, const double4_32a* en, double* out)
+{
+    const int smem = (int)sizeof(float4) * G * 4 * KB, per = 2 * KB / G;
+    PB_CUDA(c, cudaFuncSetAttribute(k_rhs_x2<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_rhs_x2<G><<<(nt + per - 1) / per, KB, smem, c->st>>>(nt, c->nc, ep, en, c->qpos, c->q, c->prm.eps_in, out);
+    PB_LAUNCH(c);
+    return PB_OK;
 }
 
 int pb_rhs_sorted(pb_ctx* c, double* bs)
@@ -190,12 +230,17 @@ int pb_rhs_sorted(pb_ctx* c, double* bs)
     const double4_32a* en = c->q2 > 1 ? c->pts_n : c->e64n;
     double* out = c->q2 > 1 ? c->yq : bs;
     pb_tic(c, PB_T_RHS);
-    if (c->prm.precision == PB_MIXED)
-        k_rhs_x2<<<(nt + 2 * KB - 1) / (2 * KB), KB, 0, c->st>>>(nt, c->nc, ep, en, c->qpos, c->q, c->prm.eps_in, out);
-    else
+    if (c->prm.precision == PB_MIXED) {
+        // four groups where one leaves the GPU short of warps (fewer than two waves of blocks) and
+        // there are charges for three of them (1,310,720 elements and 14,000 charges: 11.0 ms with one group,
+        // 11.7 with four)
+        const bool split = nt < 2 * KB * 152 * 8 && c->nc > 2 * KB;
+        if (const int rc = split ? rhs_x2<4>(c, nt, ep, en, out) : rhs_x2<1>(c, nt, ep, en, out)) return rc;
+    } else {
         k_rhs<double><<<(nt + 2 * KB - 1) / (2 * KB), KB, 0, c->st>>>(nt, c->nc, ep, en, c->qpos, c->q, c->prm.eps_in,
                                                                       out);
-    PB_LAUNCH(c);
+        PB_LAUNCH(c);
+    }
     if (c->q2 > 1) {
         int rc = pb_from_points(c, c->yq, bs, 0, c->st);
         if (rc) return rc;

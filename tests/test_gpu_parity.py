@@ -383,3 +383,21 @@ def test_scans_across_one_block_and_tiles(n):
         assert st["touching"] == sum(c * c for c in share.values()) - int((k * k).sum()) + m.nt
     finally:
         pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("nc", [1, 255, 257, 512, 513, 1025, 2100])
+def test_rhs_charge_groups(sphere3, nc):
+    # tiles of 256 charges, one group of threads up to 512 charges and four beyond, with empty and ragged
+    # last tiles. Charges of one sign inside a sphere: all terms of either half have one sign, so the
+    # FP32 sum of a tile (256 terms) is within 256 * 2^-24 = 1.5e-5 of itself
+    m, ph, _ = sphere3
+    rng = np.random.default_rng(nc)
+    R = float(np.linalg.norm(m.verts[0]))
+    m = inputs.Mesh(m.verts, m.tris, rng.uniform(-0.4, 0.4, (nc, 3)) * R, rng.uniform(0.1, 1.0, nc))
+    ctx = _ctx(m, leaf_size=48, p=4, precision=pb.PB_MIXED)
+    try:
+        b = torch.empty(2 * m.nt, device="cuda", dtype=torch.float64)
+        pb.pb_rhs(ctx, b)
+        np.testing.assert_allclose(b.cpu().numpy(), dense.rhs(m, ph), rtol=2e-5)
+    finally:
+        pb.pb_destroy(ctx)
