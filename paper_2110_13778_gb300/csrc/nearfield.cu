@@ -775,13 +775,21 @@ struct MvEnd {
     const int* order;
     double* y;
 };
+// The roundings of a row are written out: contracted as the compiler likes, the same expressions in another
+// kernel differ in the last bit, and the FP32 preconditioner, which rounds its input, carries one such bit
+// on as a whole FP32 ulp of single entries of a solution (1e-7 of its maximum).
+// f A x - A s
+__device__ __forceinline__ double mass_row(double f, double A, double x, double s)
+{
+    return __fma_rn(__dmul_rn(f, A), x, -__dmul_rn(A, s));
+}
 __device__ __forceinline__ void mv_end(const MvEnd& m, long long o, int k, double c1, double c2)
 {
     double a = m.ys[o + k], b = m.ys[o + m.nt + k];
     if (m.ep) {
         const double A = m.ep[k].w;
-        a = 0.5 * (1.0 + m.eps) * A * m.xs[o + k] - A * a;
-        b = 0.5 * (1.0 + 1.0 / m.eps) * A * m.xs[o + m.nt + k] - A * b;
+        a = mass_row(0.5 * (1.0 + m.eps), A, m.xs[o + k], a);
+        b = mass_row(0.5 * (1.0 + 1.0 / m.eps), A, m.xs[o + m.nt + k], b);
     }
     if (m.yf) {
         c1 -= m.yf[o + k];
@@ -819,8 +827,8 @@ __global__ void __launch_bounds__(32 * CORR_W) k_corrections(const int* __restri
             const int t = base + i, j = tj[t];
             const double2 a = c2[2 * (size_t)t], b = c2[2 * (size_t)t + 1];
             const double ph = m.xs[j], dph = m.xs[nt + j];
-            s1[w][i] = a.x * dph + a.y * ph;
-            s2[w][i] = b.x * dph + b.y * ph;
+            s1[w][i] = __fma_rn(a.x, dph, __dmul_rn(a.y, ph));
+            s2[w][i] = __fma_rn(b.x, dph, __dmul_rn(b.y, ph));
         }
         __syncwarp();
         for (int i = max(t0 - base, 0); i < min(t1 - base, n); ++i) {
@@ -954,9 +962,9 @@ int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
 }
 
 // Several right-hand sides: four per thread (blockIdx.y = group of four), so each correction
-// is read once per four vectors instead of once per vector. Bound: the FP64 pipe, four FMA per pair
-// and vector (16 vectors on 81,920 elements: 158 us; products added up afterwards, six operations,
-// took 236 us).
+// is read once per four vectors instead of once per vector. Bound: the FP64 pipe, six operations per
+// pair and vector (16 vectors on 81,920 elements: 236 us; chains of FMA, four operations, took 158 us, but
+// round each row otherwise, and single entries of a batched solution then move by an FP32 ulp).
 __global__ void k_corrections4(int nr, const int* __restrict__ toff, const int* __restrict__ tj,
                                const double* __restrict__ corr, MvEnd m)
 {
@@ -976,8 +984,8 @@ __global__ void k_corrections4(int nr, const int* __restrict__ toff, const int* 
             if (q < nq) {
                 const double* x = m.xs + (q0 + q) * vs;
                 const double ph = x[j], dph = x[nt + j];
-                y1[q] = fma(c0, dph, fma(c1, ph, y1[q]));
-                y2[q] = fma(c2, dph, fma(c3, ph, y2[q]));
+                y1[q] = __dadd_rn(y1[q], __fma_rn(c1, ph, __dmul_rn(c0, dph)));
+                y2[q] = __dadd_rn(y2[q], __fma_rn(c3, ph, __dmul_rn(c2, dph)));
             }
     }
 #pragma unroll
