@@ -42,11 +42,23 @@
 // which k_near64_sum adds per element in tile order: no atomics, and the product does not depend
 // on scheduling. 20,480 elements: near field 1.80 ms; 11.3 ms one direction at a time with a block of 128
 // threads per leaf of 76.
+//
+// The tiles are numbered, not listed: chunk a is the first of tiles base[a] .. base[a + 1], with the
+// chunks b >= a of its own leaf k, then those of the neighbour leaves after k in list order (pos[t]: the
+// place of neighbour entry t there; for an entry t to a leaf before k, pos[t] is the place of k in that
+// leaf's tiles). A product takes the tiles in batches of whole first chunks, of at most NEAR64_BATCH
+// tiles, so that their sums take 256 MB however large the leaves are.
+#define NEAR64_BATCH (1 << 18)
+struct Near64Tiles {
+    const long long* base;
+    const int *first, *noff, *nidx, *pos;  // first: first chunk of each leaf
+    int a0, a1;                            // the batch: its first chunks
+};
 struct Near64Src {
     double x[32], y[32], z[32], nx[32], ny[32], nz[32], phi[32], dphi[32];
     double r1[64], r2[64];  // ceil(32 / nb) groups of nb <= 32 sums: at most 63
 };
-__global__ void __launch_bounds__(256, 2) k_near64(int nt, int ntiles, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(256, 2) k_near64(int nt, const __grid_constant__ Near64Tiles q,
                                                 const int* __restrict__ chunk_leaf,
                                                 const int* __restrict__ chunk_first, const int* __restrict__ begin,
                                                 const double4_32a* __restrict__ ep, const double4_32a* __restrict__ en,
@@ -54,11 +66,37 @@ __global__ void __launch_bounds__(256, 2) k_near64(int nt, int ntiles, const int
                                                 double* __restrict__ part)
 {
     __shared__ Near64Src sh[8];
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (w >= ntiles) return;
+    const long long at = q.base[q.a0] + w;
+    if (at >= q.base[q.a1]) return;
     Near64Src& S = sh[threadIdx.x >> 5];
-    int2 t = tiles[w];
+    int2 t;  // the chunks of tile `at`
+    {
+        int lo = q.a0, hi = q.a1;  // base[lo] <= at < base[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (q.base[mid] <= at) lo = mid;
+            else hi = mid;
+        }
+        const int k = chunk_leaf[lo], own = q.first[k + 1] - lo;
+        int j = (int)(at - q.base[lo]);
+        t = make_int2(lo, lo + j);
+        if (j >= own) {
+            j -= own;
+            t.y = lo;
+            for (int e0 = q.noff[k]; e0 < q.noff[k + 1]; e0 += 32) {
+                const int e = e0 + lane, c = e < q.noff[k + 1] ? q.nidx[e] : -1;
+                const int b = c > k ? j - q.pos[e] : -1;
+                const bool here = b >= 0 && b < q.first[c + 1] - q.first[c];
+                const unsigned m = __ballot_sync(0xffffffffu, here);
+                if (m) {
+                    t.y = __shfl_sync(0xffffffffu, here ? q.first[c] + b : 0, __ffs(m) - 1);
+                    break;
+                }
+            }
+        }
+    }
     int a0 = chunk_first[t.x], b0 = chunk_first[t.y];
     int na = min(32, begin[chunk_leaf[t.x] + 1] - a0), nb = min(32, begin[chunk_leaf[t.y] + 1] - b0);
     const bool diag = t.x == t.y;
@@ -141,40 +179,60 @@ __global__ void __launch_bounds__(256, 2) k_near64(int nt, int ntiles, const int
 }
 
 // One warp per chunk: y1 = 1/2 (1 + eps) A phi - A acc1, y2 = 1/2 (1 + 1/eps) A dphi - A acc2 with
-// acc the tiles' sums of the chunk (list[off[c]..off[c + 1]): 2 * tile + side) in list order.
-__global__ void __launch_bounds__(256) k_near64_sum(int nt, int nchunks, const int* __restrict__ off,
-                                                    const int* __restrict__ list, const int* __restrict__ chunk_leaf,
+// acc the tiles' sums of the chunk in tile order. ys carries acc from batch to batch (start: the first
+// batch, end: the last).
+__global__ void __launch_bounds__(256) k_near64_sum(int nt, int nchunks, const __grid_constant__ Near64Tiles q,
+                                                    const int* __restrict__ chunk_leaf,
                                                     const int* __restrict__ chunk_first, const int* __restrict__ begin,
                                                     const double4_32a* __restrict__ ep, const double* __restrict__ part,
-                                                    const double* __restrict__ xs, double eps, double* __restrict__ ys)
+                                                    const double* __restrict__ xs, double eps, bool start, bool end,
+                                                    double* __restrict__ ys)
 {
-    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= nchunks) return;
-    const int k = chunk_first[c] + lane;
-    double a1 = 0.0, a2 = 0.0;
-#pragma unroll 4
-    for (int t = off[c]; t < off[c + 1]; ++t) {
-        const double* p = part + (size_t)list[t] * 64;
+    const int leaf = chunk_leaf[c], k = chunk_first[c] + lane;
+    const bool act = k < begin[leaf + 1];
+    const long long t0 = q.base[q.a0];
+    double a1 = start || !act ? 0.0 : ys[k], a2 = start || !act ? 0.0 : ys[nt + k];
+    auto add = [&](long long tile, int side) {
+        const double* p = part + (size_t)(tile - t0) * 128 + side * 64;
         a1 += p[lane];
         a2 += p[32 + lane];
+    };
+    for (int e = q.noff[leaf]; e < q.noff[leaf + 1]; ++e) {
+        const int l = q.nidx[e];
+        if (l > leaf) continue;
+        // as second chunk: of the chunks of a leaf before, and of the own leaf's chunks before this one
+        const int own = q.first[l + 1], to = min(l == leaf ? c : own, q.a1);
+        const int at = l == leaf ? c : own + q.pos[e] + c - q.first[leaf];
+#pragma unroll 4
+        for (int a = max(q.first[l], q.a0); a < to; ++a) add(q.base[a] + (at - a), 1);
     }
-    if (k >= begin[chunk_leaf[c] + 1]) return;
-    const double A = ep[k].w;
-    ys[k] = 0.5 * (1.0 + eps) * A * xs[k] - A * a1;
-    ys[nt + k] = 0.5 * (1.0 + 1.0 / eps) * A * xs[nt + k] - A * a2;
+    if (c >= q.a0 && c < q.a1) {
+        const long long t1 = q.base[c + 1];
+#pragma unroll 4
+        for (long long t = q.base[c]; t < t1; ++t) add(t, 0);
+    }
+    if (!act) return;
+    if (end) {
+        const double A = ep[k].w;
+        a1 = 0.5 * (1.0 + eps) * A * xs[k] - A * a1;
+        a2 = 0.5 * (1.0 + 1.0 / eps) * A * xs[nt + k] - A * a2;
+    }
+    ys[k] = a1;
+    ys[nt + k] = a2;
 }
 
-// chunks, pair tiles, each chunk's list of tile sums, and the tiles' sums
+// chunks, the numbering of the pair tiles, its batches, and the sums of one batch
 static int near64_setup(pb_ctx* c)
 {
     const PbLevel& lv = c->lev[c->L];
     const std::vector<int>&b = c->h_leaf_begin, &no = c->h_near_off, &ni = c->h_near_idx;
-    std::vector<int>&cl = c->h_up_i[0], &cf = c->h_up_i[1], &lst = c->h_up_i[4], &off = c->h_up_i[5];
-    std::vector<int2>& tl = c->h_up_i2;
+    std::vector<int>&cl = c->h_up_i[0], &cf = c->h_up_i[1], &pos = c->h_up_i[4], &first = c->h_up_i[5];
+    std::vector<long long>& base = c->h_up_l64;
     cl.clear();
     cf.clear();
-    tl.clear();
-    std::vector<int> first(lv.ncl + 1, 0);
+    first.assign(lv.ncl + 1, 0);
     for (int k = 0; k < lv.ncl; ++k) {
         for (int s = b[k]; s < b[k + 1]; s += 32) {
             cl.push_back(k);
@@ -183,41 +241,44 @@ static int near64_setup(pb_ctx* c)
         first[k + 1] = (int)cl.size();
     }
     c->nchunks = (int)cl.size();
-    for (int k = 0; k < lv.ncl; ++k)
-        for (int a = first[k]; a < first[k + 1]; ++a)
-            for (int t = no[k]; t < no[k + 1]; ++t) {
-                const int c2 = ni[t];
-                if (c2 < k) continue;
-                for (int q = c2 == k ? a : first[c2]; q < first[c2 + 1]; ++q) tl.push_back(make_int2(a, q));
+    pos.assign(ni.size(), 0);
+    base.assign(1, 0);
+    for (int k = 0; k < lv.ncl; ++k) {
+        int after = 0;  // chunks of the neighbour leaves after k
+        for (int t = no[k]; t < no[k + 1]; ++t)
+            if (ni[t] > k) {
+                pos[t] = after;
+                after += first[ni[t] + 1] - first[ni[t]];
             }
-    if (tl.size() > 0x3fffffff) return pb_fail(c, PB_ERR_NOMEM, "near setup: too many pair tiles");
-    off.assign(c->nchunks + 1, 0);
-    for (const int2& t : tl) {
-        ++off[t.x + 1];
-        if (t.y != t.x) ++off[t.y + 1];
+        for (int a = first[k]; a < first[k + 1]; ++a) base.push_back(base.back() + (first[k + 1] - a) + after);
     }
-    for (int k = 0; k < c->nchunks; ++k) off[k + 1] += off[k];
-    lst.resize(off[c->nchunks]);
-    std::vector<int> at(off.begin(), off.end() - 1);
-    for (size_t t = 0; t < tl.size(); ++t) {
-        lst[at[tl[t].x]++] = (int)(2 * t);
-        if (tl[t].y != tl[t].x) lst[at[tl[t].y]++] = (int)(2 * t + 1);
+    for (int k = 0; k < lv.ncl; ++k)
+        for (int t = no[k]; t < no[k + 1]; ++t)
+            if (ni[t] < k)
+                for (int u = no[ni[t]]; u < no[ni[t] + 1]; ++u)  // (neighbours are mutual)
+                    if (ni[u] == k) pos[t] = pos[u];
+    std::vector<int>& cut = c->near64_cut;
+    cut.assign(1, 0);
+    long long most = 0;
+    for (int a = 0; a < c->nchunks; ++a) {
+        if (a > cut.back() && base[a + 1] - base[cut.back()] > NEAR64_BATCH) cut.push_back(a);
+        most = std::max(most, base[a + 1] - base[cut.back()]);
     }
-    c->near_nitems = (int)tl.size();
+    cut.push_back(c->nchunks);
     c->chunk_leaf = (int*)pb_alloc(c, sizeof(int) * cl.size());
     c->chunk_first = (int*)pb_alloc(c, sizeof(int) * cf.size());
-    c->near_tiles2 = (int2*)pb_alloc(c, sizeof(int2) * tl.size());
-    c->near_off = (int*)pb_alloc(c, sizeof(int) * off.size());
-    c->near_list = (int*)pb_alloc(c, sizeof(int) * lst.size());
-    c->near_part = (double*)pb_alloc(c, sizeof(double) * 128 * tl.size());
-    if (!c->chunk_leaf || !c->chunk_first || !c->near_tiles2 || !c->near_off || !c->near_list || !c->near_part)
+    c->near64_first = (int*)pb_alloc(c, sizeof(int) * first.size());
+    c->near64_pos = (int*)pb_alloc(c, sizeof(int) * pos.size());
+    c->near64_base = (long long*)pb_alloc(c, sizeof(long long) * base.size());
+    c->near_part = (double*)pb_alloc(c, sizeof(double) * 128 * (size_t)most);
+    if (!c->chunk_leaf || !c->chunk_first || !c->near64_first || !c->near64_pos || !c->near64_base || !c->near_part)
         return pb_fail(c, PB_ERR_NOMEM, "near setup: out of memory");
     auto up = [&](void* d, const void* h, size_t n) { return cudaMemcpyAsync(d, h, n, cudaMemcpyHostToDevice, c->st); };
     PB_CUDA(c, up(c->chunk_leaf, cl.data(), sizeof(int) * cl.size()));
     PB_CUDA(c, up(c->chunk_first, cf.data(), sizeof(int) * cf.size()));
-    PB_CUDA(c, up(c->near_tiles2, tl.data(), sizeof(int2) * tl.size()));
-    PB_CUDA(c, up(c->near_off, off.data(), sizeof(int) * off.size()));
-    PB_CUDA(c, up(c->near_list, lst.data(), sizeof(int) * lst.size()));
+    PB_CUDA(c, up(c->near64_first, first.data(), sizeof(int) * first.size()));
+    PB_CUDA(c, up(c->near64_pos, pos.data(), sizeof(int) * pos.size()));
+    PB_CUDA(c, up(c->near64_base, base.data(), sizeof(long long) * base.size()));
     return PB_OK;
 }
 
@@ -949,13 +1010,22 @@ int pb_near_apply(pb_ctx* c, const double* xs, double* ys)
             c->nt, c->near_nitems, c->near_items, c->near_tiles, c->chunk_leaf, c->chunk_first, lv.begin, c->near_sp,
             c->near_sn, c->e32l, eps, c->prm.kappa, ys);
     } else {
-        k_near64<<<(unsigned)(((long long)c->near_nitems * 32 + 255) / 256), 256, 0, c->st>>>(
-            c->nt, c->near_nitems, c->near_tiles2, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p, c->e64n, xs, eps,
-            c->prm.kappa, c->near_part);
-        PB_LAUNCH(c);
-        k_near64_sum<<<(unsigned)(((long long)c->nchunks * 32 + 255) / 256), 256, 0, c->st>>>(
-            c->nt, c->nchunks, c->near_off, c->near_list, c->chunk_leaf, c->chunk_first, lv.begin, c->e64p,
-            c->near_part, xs, eps, ys);
+        Near64Tiles q = {c->near64_base, c->near64_first, lv.near_off, lv.near_idx, c->near64_pos, 0, 0};
+        const std::vector<int>& cut = c->near64_cut;
+        const std::vector<long long>& base = c->h_up_l64;
+        for (size_t i = 0; i + 1 < cut.size(); ++i) {
+            q.a0 = cut[i];
+            q.a1 = cut[i + 1];
+            const long long tiles = base[q.a1] - base[q.a0];
+            k_near64<<<(unsigned)((tiles + 7) / 8), 256, 0, c->st>>>(c->nt, q, c->chunk_leaf, c->chunk_first, lv.begin,
+                                                                     c->e64p, c->e64n, xs, eps, c->prm.kappa, c->near_part);
+            PB_LAUNCH(c);
+            k_near64_sum<<<(c->nchunks + 7) / 8, 256, 0, c->st>>>(c->nt, c->nchunks, q, c->chunk_leaf, c->chunk_first,
+                                                                  lv.begin, c->e64p, c->near_part, xs, eps, i == 0,
+                                                                  i + 2 == cut.size(), ys);
+            PB_LAUNCH(c);
+        }
+        return PB_OK;
     }
     PB_LAUNCH(c);
     return PB_OK;

@@ -116,10 +116,11 @@ struct pb_ctx {
     double* pn_y = nullptr;
     std::vector<int> h_pn_i[3];
     std::vector<int4> h_pn_i4;
-    // FP64 near field: chunk pairs, the sums of both chunks of each, and per chunk the list of its
-    // sums (2 * tile + side)
-    int2* near_tiles2 = nullptr;
-    int *near_off = nullptr, *near_list = nullptr;
+    // FP64 near field: the numbering of the pair tiles (per first chunk, leaf and neighbour entry), the
+    // first chunks that open a batch, and the sums of one batch
+    long long* near64_base = nullptr;
+    int *near64_first = nullptr, *near64_pos = nullptr;
+    std::vector<int> near64_cut;
     double* near_part = nullptr;
     float4* near_sp = nullptr;  // (x_hi, y_hi, z_hi, A phi)
     float4* near_sn = nullptr;  // (n_x, n_y, n_z, A dphi)
@@ -142,10 +143,10 @@ struct pb_ctx {
     // those copies need no synchronisation
     std::vector<int> h_leaf_begin, h_near_off, h_near_idx;  // leaf ranges and leaf neighbour lists
     // h_up_i: [0] chunk leaf, [1] chunk first element, [2] preconditioner block ranges, [3] block
-    // ids by size class, [4] near-field pair tiles (FP64: the chunks' lists of tile sums), [5]
-    // several-vector directed tiles (FP64: the offsets of those lists)
+    // ids by size class, [4] near-field pair tiles (FP64: places of the neighbour entries),
+    // [5] several-vector directed tiles (FP64: first chunk of each leaf)
     std::vector<int> h_up_i[6];
-    std::vector<int2> h_up_i2;            // FP64 near-field pair tiles
+    std::vector<long long> h_up_l64;      // FP64 near field: first tile of each first chunk
     std::vector<int4> h_up_i4, h_up_i4m;  // near-field work items: pair tiles, directed tiles
     std::vector<long long> h_up_l;        // preconditioner block offsets
     std::vector<double> h_up_d;           // singular quadrature: Gauss-Legendre nodes and weights

@@ -401,3 +401,52 @@ def test_rhs_charge_groups(sphere3, nc):
         np.testing.assert_allclose(b.cpu().numpy(), dense.rhs(m, ph), rtol=2e-5)
     finally:
         pb.pb_destroy(ctx)
+
+
+def test_fp64_near_field_of_a_large_leaf_in_bounded_memory():
+    # one leaf of 81,920 elements: 3.3 million pair tiles, whose sums (1 KB each) are held for 262,144 tiles at
+    # a time, 256 MB beside 0.1 GB of lists and records; a few rows against the direct sum in FP64.
+    # Bar as above (1e-10)
+    V, T = inputs.icosphere(6, 30.0)
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    ctx = _ctx(m, eta0=0.8, leaf_size=10**6, p=2, qs=2, precision=pb.PB_FP64, precond=pb.PB_PRECOND_DIAG)
+    try:
+        assert pb.pb_get_tree_stats(ctx)["max_leaf"] == m.nt
+        assert free0 - torch.cuda.mem_get_info()[0] < 1 << 30
+        x = _dev(inputs.random_density(m.nt, 3))
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        pb.pb_matvec_part(ctx, x, y, 1)
+        # rows of elements that touch nothing in the density's support, against the sum over it
+        P = _dev(V[T].mean(1))
+        E1, E2 = _dev(V[T[:, 1]] - V[T[:, 0]]), _dev(V[T[:, 2]] - V[T[:, 0]])
+        N = torch.linalg.cross(E1, E2)
+        A = N.norm(dim=1) / 2
+        N = N / (2 * A[:, None])
+        far = P[:, 2] > 0
+        xs = x.view(2, -1) * far  # support: the upper half
+        pb.pb_matvec_part(ctx, xs.reshape(-1).contiguous(), z, 1)
+        rows = torch.nonzero(P[:, 2] < -1.0).ravel()[:: m.nt // 97]
+        d = P[rows, None, :] - P[None]
+        r2 = (d * d).sum(-1)
+        r = r2.sqrt()
+        t = KAP * r
+        e = torch.exp(-t)
+        xd, yd = (N[rows, None] * d).sum(-1), (N[None] * d).sum(-1)
+        nn = N[rows] @ N.T
+        ph, dph = (A * xs[0])[None], (A * xs[1])[None]
+        g3 = 1 / r**3
+        k1, k2 = -torch.expm1(-t) / r, yd * g3 * (80.0 * e * (1 + t) - 1)
+        k3 = -xd * g3 * (1 - e * (1 + t) / 80.0)
+        k4 = g3 * ((3 - e * (3 + 3 * t + t * t)) * xd * yd / r2 - (1 - e * (1 + t)) * nn)
+        on = far[None]
+        s1 = torch.where(on, k1 * dph + k2 * ph, 0.0).sum(1) / (4 * np.pi)
+        s2 = torch.where(on, k3 * dph + k4 * ph, 0.0).sum(1) / (4 * np.pi)
+        want = torch.stack([-A[rows] * s1, -A[rows] * s2])
+        assert _rel(z.view(2, -1)[:, rows].cpu().numpy(), want.cpu().numpy()) < 1e-10
+        # linear: the product of both halves' densities adds up
+        pb.pb_matvec_part(ctx, (x.view(2, -1) * ~far).reshape(-1).contiguous(), xs.view(-1), 1)
+        assert _rel((xs.view(-1) + z).cpu().numpy(), y.cpu().numpy()) < 1e-12
+    finally:
+        pb.pb_destroy(ctx)
