@@ -697,10 +697,10 @@ __global__ void k_near_dens(int nt, const float4* __restrict__ e32p, const int* 
 // atomics, so that items of one target chunk may run on different warps. Each tile's source
 // records and its NR densities are staged in shared memory by coalesced loads (one per lane
 // and record), so the pair loop reads them as shared-memory broadcasts. Two densities (r, r + 1) are
-// the halves of packed FP32 pairs in the four FMAs per density. A tile's FP32 sums go into
-// float-float accumulators (an exact two-sum, 2^-48): with FP64 ones (a conversion and an addition per
-// value, at 1/64 of the FP32 rate) the FP64 pipe was 55 % busy and held the loop up. 81,920 elements,
-// 16 densities: 870 -> 635 us.
+// the halves of packed FP32 pairs in the four FMAs per density. A tile's FP32 sums go into FP64
+// accumulators, a conversion and an addition per value at 1/64 of the FP32 rate: float-float ones (2^-48)
+// save 70 us of 2360 per product of 16 densities on 81,920 elements, but are less than FP64 and change
+// last bits of products; conversions by integer operations gain nothing (2390 us).
 template <int NR>
 struct NearM {
     static constexpr int H = (NR + 1) / 2;  // pairs of densities
@@ -735,14 +735,6 @@ __device__ __forceinline__ void near_m_tile(const float4 tp, const float4 tn, co
     }
 }
 
-// (hi, lo) += s, per half
-__device__ __forceinline__ void x2_ff_acc(f2x& hi, f2x& lo, f2x s)
-{
-    const f2x t = x2_add(hi, s), bb = x2_sub(t, hi);
-    lo = x2_add(lo, x2_add(x2_sub(hi, x2_sub(t, bb)), x2_sub(s, bb)));
-    hi = t;
-}
-
 template <int NR>
 __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const int4* __restrict__ items,
                                                     const int* __restrict__ tiles, const int* __restrict__ chunk_leaf,
@@ -762,7 +754,7 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
     float4* s_n = (float4*)nsm + 256 + wi * 32;
     float4* s_l = (float4*)nsm + 512 + wi * 32;
     float4* s_d = (float4*)nsm + 768 + wi * H * 32;                           // (x_r, x_r+1, y_r, y_r+1)
-    f2x* s_acc = (f2x*)((float4*)nsm + 768 + 8 * H * 32) + wi * 4 * H * 32;  // [4 h + (hi1, lo1, hi2, lo2)][lane]
+    double* s_acc = (double*)((float4*)nsm + 768 + 8 * H * 32) + wi * 4 * H * 32;  // [density][half of the row][lane]
     if (w >= nitems) return;
     const int4 item = items[w];
     const int c = chunk_leaf[item.x];
@@ -772,7 +764,7 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
     const float4 tp = sp[kk], tn = sn[kk], tl = sl[kk];
     const float eps = (float)eps_d, inv_eps = (float)(1.0 / eps_d), kappa = (float)kappa_d;
 #pragma unroll
-    for (int r = 0; r < 4 * H; ++r) s_acc[r * 32 + lane] = 0ull;
+    for (int r = 0; r < 4 * H; ++r) s_acc[r * 32 + lane] = 0.0;
     for (int ti = item.y; ti < item.z; ++ti) {
         const int tv = tiles[ti], cb = tv & (NEAR_FAR - 1);
         const int sb = chunk_first[cb], se = min(sb + 32, begin[chunk_leaf[cb] + 1]);
@@ -798,30 +790,22 @@ __global__ void __launch_bounds__(256, 2) k_near32m(int nt, int nitems, const in
         else near_m_tile<NR, false>(tp, tn, tl, s_p, s_n, s_l, s_d, nb, k - sb, eps, inv_eps, kappa, s1, s2);
 #pragma unroll
         for (int h = 0; h < H; ++h) {
-            f2x* a = s_acc + 4 * h * 32 + lane;
-            x2_ff_acc(a[0], a[32], s1[h]);
-            x2_ff_acc(a[64], a[96], s2[h]);
+            double* a = s_acc + 4 * h * 32 + lane;
+            float v[4];
+            x2_unpack(s1[h], v[0], v[2]);
+            x2_unpack(s2[h], v[1], v[3]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[32 * u] += (double)(v[u]);
         }
     }
     // densities beyond nvalid are padding of the group (finite, unused): only nvalid are added
     if (act)
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-            const f2x* a = s_acc + 4 * h * 32 + lane;
-            float h1[2], l1[2], h2[2], l2[2];
-            x2_unpack(a[0], h1[0], h1[1]);
-            x2_unpack(a[32], l1[0], l1[1]);
-            x2_unpack(a[64], h2[0], h2[1]);
-            x2_unpack(a[96], l2[0], l2[1]);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int r = 2 * h + u;
-                if (r < nvalid) {
-                    atomicAdd(&ys[2LL * nt * r + k], (double)h1[u] + (double)l1[u]);
-                    atomicAdd(&ys[2LL * nt * r + nt + k], (double)h2[u] + (double)l2[u]);
-                }
+        for (int r = 0; r < NR; ++r)
+            if (r < nvalid) {
+                atomicAdd(&ys[2LL * nt * r + k], s_acc[2 * r * 32 + lane]);
+                atomicAdd(&ys[2LL * nt * r + nt + k], s_acc[(2 * r + 1) * 32 + lane]);
             }
-        }
 }
 
 // What ends a product. ep: ys holds the mixed near field's bare sums, which become

@@ -450,3 +450,35 @@ def test_fp64_near_field_of_a_large_leaf_in_bounded_memory():
         assert _rel((xs.view(-1) + z).cpu().numpy(), y.cpu().numpy()) < 1e-12
     finally:
         pb.pb_destroy(ctx)
+
+
+def test_several_vectors_add_tiles_in_fp64():
+    # 248 elements in one leaf: every row's eight tiles are one work item, summed in FP64. Densities u
+    # on the first chunk and w = 2^-k on the third are evaluated alone and together, so that the rows of a
+    # third place are sums of the same two FP32 tile sums: y(u + w) = y(u) + y(w) up to five roundings, of
+    # the sum, of the three rows and of the addition below, each 2^-53 of the largest value
+    V, T = inputs.icosphere(3, 4.0)
+    T = T[:248]
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    ctx = _ctx(m, eta0=0.8, leaf_size=1000, p=2, precision=pb.PB_MIXED, precond=pb.PB_PRECOND_DIAG)
+    try:
+        order = pb.pb_get_tree(ctx, m.nt)[1]
+        u, w = np.zeros(m.nt), np.zeros(m.nt)
+        u[order[:32]] = inputs.random_density(m.nt, 1)[:32]
+        w[order[64:96]] = inputs.random_density(m.nt, 2)[:32]
+        near = np.isin(T, T[np.concatenate([order[:32], order[64:96]])]).any(1)  # the corrections' rows
+        rows = np.tile(~near, 2)
+        assert rows.sum() > 150
+        X = []
+        for k in (8, 16, 20, 24, 28):
+            for a, b in ((u, 0 * w), (0 * u, w * 2.0**-k), (u, w * 2.0**-k)):
+                X.append(np.concatenate([a + b, 0.5 * a - b]))
+        X = _dev(np.stack(X + [X[0]]))
+        Y = torch.empty_like(X)
+        pb.pb_matvec_multi(ctx, X, Y)
+        Y = Y.cpu().numpy()[:, rows]
+        for a, b, c in zip(Y[0:15:3], Y[1:15:3], Y[2:15:3]):
+            big = np.maximum(np.maximum(np.abs(a), np.abs(b)), np.abs(c))
+            assert np.all(np.abs(c - (a + b)) <= 5 * 2.0**-53 * big)
+    finally:
+        pb.pb_destroy(ctx)
