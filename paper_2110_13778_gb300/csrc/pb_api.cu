@@ -61,11 +61,6 @@ static void pb_free_build(pb_ctx* c)
     c->far_nr = 1;
     c->mxs = c->mys = c->gbV = c->gbW = c->gbZ = c->gbB = c->gbpart = c->gbsmall = nullptr;
     pb_dg_drop(c);
-    c->tc_part = nullptr;
-    c->tc_nw = 0;
-    c->tc_list = nullptr;
-    c->tc_cnt = nullptr;
-    c->tc_lpart = nullptr;
     c->bE = nullptr;
     c->bE_n = 0;
     c->q2 = 1;

@@ -199,11 +199,6 @@ struct pb_ctx {
     long long dg_cnt[3] = {};
     bool dg_failed = false;           // graphs with conditional nodes cannot be built here
     long long build_gen = 0;          // incremented by every pb_build_tree / pb_mesh_upload
-    double* tc_part = nullptr;        // treecode energy: one partial per (charge, level-1 cluster)
-    long long tc_nw = 0;
-    int2* tc_list = nullptr;     // treecode energy by lists: pairs, counters, partial sums
-    int* tc_cnt = nullptr;
-    double* tc_lpart = nullptr;
     // regular rule of order q > 1: q2 = q^2 points per element, their records (tree order,
     // element-major), the leaf ranges in points and point work vectors (2 x N q2 each)
     int q2 = 1;

@@ -136,3 +136,43 @@ def test_lists_too_short_for_a_small_theta(prec, tol, nc, theta):
         assert abs(E - Ed) < tol * max(abs(Ed), scale)
     finally:
         pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [pb.PB_FP64, pb.PB_MIXED])
+@pytest.mark.parametrize("theta", [0.5, 0.15])
+def test_energy_repeats_to_the_last_bit(prec, theta):
+    # lists and sums have a fixed order, whichever kernel a batch takes
+    V, T = inputs.icosphere(5, 20.0)
+    qp, q = inputs.ball_charges(301, 17.0, 4)
+    m = inputs.Mesh(V, T, qp, q)
+    x = _dev(inputs.random_density(m.nt, 6))
+    ctx = _ctx(m, prec, 6, leaf=16)
+    try:
+        E = {pb.pb_solvation_energy_treecode(ctx, x, theta) for _ in range(12)}
+        assert len(E) == 1, E
+    finally:
+        pb.pb_destroy(ctx)
+
+
+@pytest.mark.parametrize("nc", [16384, 16384 + 5, 2 * 16384 + 3])
+def test_batches_of_charges(nc):
+    # more than 16,384 charges go in batches: at a small theta every leaf is summed directly, so the
+    # energy is the direct sum's (bars as there)
+    V, T = inputs.icosphere(2, 6.0)
+    qp, q = inputs.ball_charges(nc, 4.5, 9)
+    m = inputs.Mesh(V, T, qp, q)
+    x = _dev(inputs.random_density(m.nt, 12))
+    ctx = _ctx(m, pb.PB_FP64, 4, leaf=8)
+    try:
+        Ed = pb.pb_solvation_energy(ctx, x)
+        scale = np.abs(q).sum() * float(x.abs().max()) * 100.0
+        assert abs(pb.pb_solvation_energy_treecode(ctx, x, 1e-6) - Ed) < 1e-12 * scale
+        # and the last batch alone counts as much as any: by charge, near the direct sum
+        for part in (slice(0, 16384), slice(nc - 3, nc)):
+            w = np.zeros(nc)
+            w[part] = q[part]
+            pb.pb_set_charges(ctx, w)
+            Et, Ed = pb.pb_solvation_energy_treecode(ctx, x, 0.4), pb.pb_solvation_energy(ctx, x)
+            assert abs(Et - Ed) < 2e-3 * max(abs(Ed), 1e-3 * np.abs(w).sum())
+    finally:
+        pb.pb_destroy(ctx)
