@@ -340,14 +340,19 @@ int pb_mlp_param_count(pb_mlp* net, long long* n);
 int pb_mlp_get_params(pb_mlp* net, float* host);
 int pb_mlp_set_params(pb_mlp* net, const float* host);
 /* Y (device, n x nout FP32, row-major) = network(X) for X (device, n x nin FP32, row-major).
- * Queues the work. */
+ * Synchronises: PB_ERR_TIMEOUT if a bounded wait of a tensor-core kernel gave up (Y is then not whole). */
 int pb_mlp_forward(pb_mlp* net, const float* X, int n, float* Y);
 /* Loss and gradient of the loss for inputs X and targets T (device, n x nout FP32); loss and
  * grad (pb_mlp_param_count floats) are host pointers and may be NULL. Synchronises. */
 int pb_mlp_gradient(pb_mlp* net, const float* X, const float* T, int n, float* loss, float* grad);
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected) on the gradient of the
- * batch (X, T). loss: host pointer or NULL (NULL leaves the step queued, no sync). */
+ * batch (X, T). loss: host pointer or NULL (NULL leaves the step queued, no sync). A step whose
+ * gradient is not whole, because a bounded wait of a tensor-core kernel gave up, leaves the
+ * parameters and the moments as they are, as does every step queued after it; the next call that
+ * synchronises returns PB_ERR_TIMEOUT, after which the network is usable again. */
 int pb_mlp_train_step(pb_mlp* net, const float* X, const float* T, int n, float lr, float* loss);
+/* For tests of that path: set the flag that a wait which gave up sets. Synchronises. */
+int pb_mlp_set_wait_flag(pb_mlp* net);
 
 /* Per-element features of the learned warm start after pb_build_tree, element order,
  * F (device, nt x 18 FP32). With r the distance from the centroid to charge k: centroid minus

@@ -37,7 +37,8 @@ struct pb_mlp {
     float* part = nullptr;
     int part_n = 0;
     float* lossbuf = nullptr;  // the loss, after the gradient in G
-    int* derr = nullptr;  // after the loss: set when a bounded wait on the tensor cores gives up
+    int* derr = nullptr;  // after the loss: [0] set when a bounded wait on the tensor cores gives up, [1] the
+                          // Adam steps left out since
     float* hbuf = nullptr;  // pinned copy of G, the loss and the flag (MLP_STAGE parameters at most, else null)
     long long nparam = 0;
     int adam_t = 0;
@@ -49,7 +50,7 @@ static int mlp_fail(pb_mlp* m, int code, const char* msg)
     if (m) m->err = msg;
     return code;
 }
-static int mlp_check_err(pb_mlp* m);
+static int mlp_check_err(pb_mlp* m, float* loss = nullptr);
 
 // ---------- tcgen05 helpers ----------
 #define TC_ROWS 128
@@ -399,9 +400,15 @@ __global__ void k_sum_slices(long long n, int slices, const float* __restrict__ 
     }
 }
 
+// (err[0] set: the gradient is not whole; the step is left out and counted)
 __global__ void k_adam(long long n, float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, float lr, float b1, float b2, float c1, float c2, float eps)
+                       const float* __restrict__ g, float lr, float b1, float b2, float c1, float c2, float eps,
+                       int* __restrict__ err)
 {
+    if (err[0]) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) ++err[1];
+        return;
+    }
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         float gi = g[i];
         float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -565,11 +572,11 @@ extern "C" int pb_mlp_create(int nin, int width, int depth, int nout, unsigned l
     bool ok = cudaMalloc(&m->W, sizeof(float) * o) == cudaSuccess;
     ok &= cudaMalloc(&m->Wm, sizeof(float) * o) == cudaSuccess;
     ok &= cudaMalloc(&m->Wv, sizeof(float) * o) == cudaSuccess;
-    ok &= cudaMalloc(&m->G, sizeof(float) * (o + 2)) == cudaSuccess;
+    ok &= cudaMalloc(&m->G, sizeof(float) * (o + 3)) == cudaSuccess;
     ok &= cudaMalloc(&m->Wb, sizeof(__nv_bfloat16) * o) == cudaSuccess;
     m->lossbuf = m->G + o;
     m->derr = (int*)(m->G + o + 1);
-    ok = ok && cudaMemset(m->derr, 0, sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMemset(m->derr, 0, 2 * sizeof(int)) == cudaSuccess;
     // (without it, should the host have no pinned memory left, the copies go one by one)
     if (ok && o <= MLP_STAGE && cudaMallocHost(&m->hbuf, sizeof(float) * (o + 2)) != cudaSuccess) {
         cudaGetLastError();
@@ -842,7 +849,7 @@ extern "C" int pb_mlp_forward(pb_mlp* m, const float* X, int n, float* Y)
     if (cudaMemcpy2DAsync(Y, sizeof(float) * m->nout, m->Z, sizeof(float) * dl, sizeof(float) * m->nout, n,
                           cudaMemcpyDeviceToDevice, m->st) != cudaSuccess)
         return mlp_fail(m, PB_ERR_CUDA, "mlp: output copy failed");
-    return PB_OK;
+    return mlp_check_err(m);
 }
 
 // ---------- fused gradient: forward and backward of a tile of rows in one kernel ----------
@@ -1161,16 +1168,32 @@ static int mlp_loss_grad(pb_mlp* m, const float* X, const float* T, int n)
     return cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp gradient launch failed");
 }
 
-// PB_ERR_TIMEOUT (and the flag cleared) if a bounded wait of a tensor-core kernel gave up
-static int mlp_check_err(pb_mlp* m)
+// Synchronises; PB_ERR_TIMEOUT (the flag cleared, Adam's count of steps without those left out) if a bounded
+// wait of a tensor-core kernel gave up. loss: the loss of the last gradient, or nullptr
+static int mlp_check_err(pb_mlp* m, float* loss)
 {
-    int herr = 0;
-    if (cudaMemcpyAsync(&herr, m->derr, sizeof(int), cudaMemcpyDeviceToHost, m->st) != cudaSuccess ||
+    struct {
+        float loss;
+        int err, skipped;
+    } h = {};
+    if (cudaMemcpyAsync(&h, m->lossbuf, sizeof(h), cudaMemcpyDeviceToHost, m->st) != cudaSuccess ||
         cudaStreamSynchronize(m->st) != cudaSuccess)
         return mlp_fail(m, PB_ERR_CUDA, "mlp: sync failed");
-    if (!herr) return PB_OK;
-    cudaMemsetAsync(m->derr, 0, sizeof(int), m->st);
+    if (loss) *loss = h.loss;
+    if (!h.err) return PB_OK;
+    m->adam_t -= h.skipped;
+    cudaMemsetAsync(m->derr, 0, 2 * sizeof(int), m->st);
     return mlp_fail(m, PB_ERR_TIMEOUT, "mlp: a bounded wait on the tensor cores gave up");
+}
+
+extern "C" int pb_mlp_set_wait_flag(pb_mlp* m)
+{
+    if (!m) return PB_ERR_ARG;
+    const int one = 1;
+    if (cudaMemcpyAsync(m->derr, &one, sizeof(int), cudaMemcpyHostToDevice, m->st) != cudaSuccess ||
+        cudaStreamSynchronize(m->st) != cudaSuccess)
+        return mlp_fail(m, PB_ERR_CUDA, "mlp: copy failed");
+    return PB_OK;
 }
 
 extern "C" int pb_mlp_gradient(pb_mlp* m, const float* X, const float* T, int n, float* loss, float* grad_host)
@@ -1205,11 +1228,9 @@ extern "C" int pb_mlp_train_step(pb_mlp* m, const float* X, const float* T, int 
     m->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     float c1 = 1.f - powf(b1, (float)m->adam_t), c2 = 1.f - powf(b2, (float)m->adam_t);
-    k_adam<<<grid1(m->nparam), 256, 0, m->st>>>(m->nparam, m->W, m->Wm, m->Wv, m->G, lr, b1, b2, c1, c2, 1e-8f);
-    if (loss && cudaMemcpyAsync(loss, m->lossbuf, sizeof(float), cudaMemcpyDeviceToHost, m->st) != cudaSuccess)
-        return mlp_fail(m, PB_ERR_CUDA, "mlp: copy failed");
-    if (loss && cudaStreamSynchronize(m->st) != cudaSuccess) return mlp_fail(m, PB_ERR_CUDA, "mlp: sync failed");
-    return cudaGetLastError() == cudaSuccess ? PB_OK : mlp_fail(m, PB_ERR_CUDA, "mlp: launch failed");
+    k_adam<<<grid1(m->nparam), 256, 0, m->st>>>(m->nparam, m->W, m->Wm, m->Wv, m->G, lr, b1, b2, c1, c2, 1e-8f, m->derr);
+    if (cudaGetLastError() != cudaSuccess) return mlp_fail(m, PB_ERR_CUDA, "mlp: launch failed");
+    return loss ? mlp_check_err(m, loss) : PB_OK;
 }
 
 // ---------- features of the learned warm start ----------

@@ -28,7 +28,8 @@ EXPORTS = [
     "pb_get_tree_stats", "pb_get_tree", "pb_matvec_part", "pb_set_timing", "pb_get_timing",
     "pb_get_launch_count", "pb_solvation_energy_noalloc", "pb_solve_states",
     "pb_mlp_create", "pb_mlp_destroy", "pb_mlp_last_error", "pb_mlp_param_count", "pb_mlp_get_params",
-    "pb_mlp_set_params", "pb_mlp_forward", "pb_mlp_gradient", "pb_mlp_train_step", "pb_features",
+    "pb_mlp_set_params", "pb_mlp_forward", "pb_mlp_gradient", "pb_mlp_train_step", "pb_mlp_set_wait_flag",
+    "pb_features",
     "pb_learned_guess", "pb_measure_alu_peaks", "pb_autotune", "pb_matvec_multi", "pb_get_graph_launches",
     "pb_solvation_energy_treecode", "pb_batch_solve_states",
 ]
@@ -122,6 +123,7 @@ def lib():
         L.pb_mlp_forward.argtypes = [vp, vp, c_int, vp]
         L.pb_mlp_gradient.argtypes = [vp, vp, vp, c_int, fp, fp]
         L.pb_mlp_train_step.argtypes = [vp, vp, vp, c_int, ctypes.c_float, fp]
+        L.pb_mlp_set_wait_flag.argtypes = [vp]
         L.pb_features.argtypes = [vp, vp, vp, vp, dp]
         L.pb_learned_guess.argtypes = [vp, vp, vp]
         L.pb_measure_alu_peaks.argtypes = [vp, dp, dp]
@@ -397,6 +399,11 @@ def pb_mlp_train_step(net, X, T, lr=1e-3, want_loss=True):
     _mcheck(net, lib().pb_mlp_train_step(net, _ptr(X), _ptr(T), int(X.shape[0]), lr,
                                          ctypes.byref(loss) if want_loss else None))
     return loss.value if want_loss else None
+
+
+def pb_mlp_set_wait_flag(net):
+    """For tests: the state after a tensor-core kernel's bounded wait gave up."""
+    _mcheck(net, lib().pb_mlp_set_wait_flag(net))
 
 
 def pb_features(ctx, F, x=None, T=None):

@@ -147,6 +147,38 @@ def test_adam_step_matches_oracle(net):
         w64 = wg.copy()  # follow the GPU's FP32 weights
 
 
+@pytest.mark.parametrize("shape", [(18, 128, 3, 2), (5, 64, 2, 3)])  # fused, layer by layer
+def test_steps_are_left_out_when_a_wait_gave_up(shape):
+    # the flag of a bounded wait, set by the host: no step may touch the parameters or the moments, the next
+    # call that synchronises says so, and training then goes on as if the steps had not been asked for
+    X = torch.randn((300, shape[0]), device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    T = torch.randn((300, shape[3]), device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    end = []
+    for fail in (False, True):
+        h = pb.pb_mlp_create(*shape, seed=11)
+        try:
+            pb.pb_mlp_train_step(h, X, T, 1e-3)
+            before = pb.pb_mlp_get_params(h)
+            if fail:
+                pb.pb_mlp_set_wait_flag(h)
+                pb.pb_mlp_train_step(h, X, T, 1e-3, want_loss=False)
+                with pytest.raises(pb.PBError) as e:
+                    pb.pb_mlp_train_step(h, X, T, 1e-3)
+                assert e.value.code == pb.PB_ERR_TIMEOUT
+                assert np.array_equal(pb.pb_mlp_get_params(h), before)
+                pb.pb_mlp_set_wait_flag(h)
+                with pytest.raises(pb.PBError) as e:
+                    pb.pb_mlp_forward(h, X, torch.empty_like(T))
+                assert e.value.code == pb.PB_ERR_TIMEOUT
+            for _ in range(2):
+                pb.pb_mlp_train_step(h, X, T, 1e-3)
+            end.append(pb.pb_mlp_get_params(h))
+            assert not np.array_equal(end[-1], before)
+        finally:
+            pb.pb_mlp_destroy(h)
+    assert np.array_equal(end[0], end[1])
+
+
 def test_training_reduces_loss(net):
     rng = np.random.default_rng(8)
     X = rng.uniform(-1, 1, (8192, 18)).astype(np.float32)
