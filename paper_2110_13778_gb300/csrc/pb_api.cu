@@ -386,10 +386,21 @@ static int matvec_parts(pb_ctx* c, const double* xin, double* xs, double* ys, do
 {
     int rc;
     const int n = c->nt;
-    if (c->q2 > 1 && nr > 1) {  // the regular rule of order > 1 works one vector at a time
+    if (c->q2 > 1 && nr > 1) {
+        // the regular rule of order > 1 works one vector at a time; the caller's are all read before the
+        // first result is written (they may overlap)
+        if (xin) {
+            k_gather<<<dim3((n + 255) / 256, nr), 256, 0, c->st>>>(n, c->order, xin, xs);
+            PB_LAUNCH(c);
+        }
+        double* yt = xin ? ys : y;
         for (int r = 0; r < nr; ++r) {
             const long long o = 2LL * n * r;
-            if ((rc = matvec_parts(c, xin ? xin + o : nullptr, xs + o, ys + o, y + o, 1, which))) return rc;
+            if ((rc = matvec_parts(c, nullptr, xs + o, ys + o, yt + o, 1, which))) return rc;
+        }
+        if (xin) {
+            k_scatter<<<dim3((n + 255) / 256, nr), 256, 0, c->st>>>(n, c->order, ys, y);
+            PB_LAUNCH(c);
         }
         return PB_OK;
     }
@@ -497,7 +508,10 @@ extern "C" int pb_precond_apply(pb_ctx* c, const double* r, double* z)
     PB_ALIVE(c);
     if (!c->built) return pb_fail(c, PB_ERR_STATE, "precond before build_tree");
     if (!r || !z || r == z) return pb_fail(c, PB_ERR_ARG, "precond: bad arguments");
-    if (pb_precond_apply_element(c, r, z)) {
+    // (in one launch the blocks read r while others write z: vectors that overlap go by way of copies)
+    const size_t nu = c->prm.basis == PB_BASIS_LINEAR ? c->nv : c->nt;
+    const bool apart = r + 2 * nu <= z || z + 2 * nu <= r;
+    if (apart && pb_precond_apply_element(c, r, z)) {
         PB_CUDA(c, cudaGetLastError());
         return PB_OK;
     }

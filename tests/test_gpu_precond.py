@@ -8,7 +8,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2110_13778_gb300 import molecules, pb  # noqa: E402
+from paper_2110_13778_gb300 import inputs, molecules, pb  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -73,3 +73,29 @@ def test_pc_block_rejected_out_of_range():
     for b in (4, 97):
         with pytest.raises(pb.PBError):
             pb.pb_create(pb.params(pc_block=b))
+
+
+@pytest.mark.parametrize("prec", [pb.PB_MIXED, pb.PB_FP64])
+@pytest.mark.parametrize("shift", [1, 1000])
+def test_overlapping_vectors(prec, shift):
+    # r and z may share memory (not begin at the same place): r is read before z is written. 20,480
+    # elements make more blocks than run at once
+    V, T = inputs.icosphere(5, 20.0)
+    ctx = pb.pb_create(pb.params(eps_in=1.0, eps_out=80.0, kappa=0.1257, eta0=0.8, leaf_size=16, p=2, qs=2,
+                                 precision=prec, precond=pb.PB_PRECOND_BLOCK, singular=pb.PB_SINGULAR_FF))
+    try:
+        pb.pb_mesh_upload(ctx, V, T, np.zeros((1, 3)), np.ones(1))
+        pb.pb_build_tree(ctx)
+        n = 2 * T.shape[0]
+        r = torch.randn(n, device="cuda", dtype=torch.float64, generator=torch.Generator("cuda").manual_seed(3))
+        want = torch.empty_like(r)
+        pb.pb_precond_apply(ctx, r, want)
+        for zfirst in (False, True):
+            buf = torch.empty(n + shift, device="cuda", dtype=torch.float64)
+            a, b = buf[:n], buf[shift:]
+            rr, z = (b, a) if zfirst else (a, b)
+            rr.copy_(r)
+            pb.pb_precond_apply(ctx, rr, z)
+            assert torch.equal(z, want)
+    finally:
+        pb.pb_destroy(ctx)

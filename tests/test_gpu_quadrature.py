@@ -143,3 +143,19 @@ def test_batched_states_need_order_one(sphere):
         assert all(i.status == pb.PB_OK for i in infos)
     finally:
         pb.pb_destroy(ctx)
+
+
+def test_several_vectors_that_overlap(sphere):
+    # every vector is read before the first result is written
+    ctx = _ctx(sphere, 2, eta0=0.8, leaf_size=40, p=4, precision=pb.PB_MIXED, precond=pb.PB_PRECOND_DIAG)
+    try:
+        n, nr = 2 * sphere.nt, 3
+        X = torch.randn((nr, n), device="cuda", dtype=torch.float64, generator=torch.Generator("cuda").manual_seed(4))
+        want = torch.empty_like(X)
+        pb.pb_matvec_multi(ctx, X, want)
+        buf = torch.empty((nr + 1, n), device="cuda", dtype=torch.float64)
+        buf[:nr].copy_(X)
+        pb.pb_matvec_multi(ctx, buf[:nr], buf[1:])
+        assert torch.equal(buf[1:], want)
+    finally:
+        pb.pb_destroy(ctx)
