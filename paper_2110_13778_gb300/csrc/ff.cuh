@@ -8,7 +8,9 @@
 // cheaper than the FP64 instruction it replaces, at ~1e-14 relative accuracy.
 //
 // These helpers need IEEE FP32 semantics: no fast-math, no flush-to-zero assumptions on the
-// error terms (the build uses neither). The exponent range is FP32's.
+// error terms (the build uses neither). Products are written as __fmul_rn, which the compiler may not
+// contract into the sum that follows: the error-free transformations hold, and two instantiations of a
+// kernel give the same bits. The exponent range is FP32's.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -62,7 +64,7 @@ __device__ __forceinline__ ff ff_add_f(ff a, float b)
 // a b, relative error ~2^-46
 __device__ __forceinline__ ff ff_mul(ff a, ff b)
 {
-    float p = a.h * b.h;
+    float p = __fmul_rn(a.h, b.h);
     float e = fmaf(a.h, b.h, -p);
     e = fmaf(a.h, b.l, e);
     e = fmaf(a.l, b.h, e);
@@ -71,7 +73,7 @@ __device__ __forceinline__ ff ff_mul(ff a, ff b)
 
 __device__ __forceinline__ ff ff_mul_f(ff a, float b)
 {
-    float p = a.h * b;
+    float p = __fmul_rn(a.h, b);
     float e = fmaf(a.h, b, -p);
     e = fmaf(a.l, b, e);
     return ff_fast_two_sum(p, e);
@@ -79,22 +81,21 @@ __device__ __forceinline__ ff ff_mul_f(ff a, float b)
 
 __device__ __forceinline__ ff ff_sqr(ff a)
 {
-    float p = a.h * a.h;
+    float p = __fmul_rn(a.h, a.h);
     float e = fmaf(a.h, a.h, -p);
-    e = fmaf(2.0f * a.h, a.l, e);
+    e = fmaf(__fmul_rn(2.0f, a.h), a.l, e);
     return ff_fast_two_sum(p, e);
 }
-
-// a b + c
-__device__ __forceinline__ ff ff_fma(ff a, ff b, ff c) { return ff_add(ff_mul(a, b), c); }
 
 // 1 / sqrt(a) for a > 0: the FP32 estimate and one Newton step y + y (1 - a y^2) / 2, with
 // the residual 1 - a y^2 formed in float-float (its leading bits cancel exactly).
 __device__ __forceinline__ ff ff_rsqrt(ff a)
 {
     float y = rsqrtf(a.h);
-    float p = y * y;
+    float p = __fmul_rn(y, y);
     ff y2 = {p, fmaf(y, y, -p)};
     ff r = ff_add_f(ff_neg(ff_mul(a, y2)), 1.0f);
-    return ff_fast_two_sum(y, 0.5f * y * r.h);
+    // y + t r, and what that rounding drops
+    const float t = __fmul_rn(0.5f, y), s = fmaf(t, r.h, y);
+    return {s, fmaf(t, r.h, -(s - y))};
 }
