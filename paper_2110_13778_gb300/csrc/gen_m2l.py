@@ -4,7 +4,7 @@ For a fixed order P the MtL sum of eqcoeff, written as
     a! lam^a = sum_{|a| + |b| <= P} D^{a+b} G(d) * M^b,   M^b = (-1)^|b| m^b / b!,
 has a fixed set of (gamma = a + b, a, b) triples. Emitting them as explicit statements lets
 the compiler keep the local coefficients in registers. M2LBody<P, W> (FP64 kernel) handles one of
-NBODY[P] sets of multi-indices a with equal FMA counts (at most 42 coefficients, so that a set's
+NBODY[P] sets of multi-indices a with equal FMA counts (at most 43 coefficients, so that a set's
 accumulators fit in registers), walks gamma in layout order, loads D^gamma from the interleaved
 slot layout (Dl[gamma * 32]) in groups of GROUP so that several loads are in flight before their
 values are used, and reads the scaled moments from shared memory (Ms[b * 33]) for every FMA

@@ -866,7 +866,7 @@ extern "C" int pb_mlp_forward(pb_mlp* m, const float* X, int n, float* Y)
 // 128 contiguous bytes per warp (by rows, each lane's stores would go to a line of their own),
 // and is stored while the next layer's products run (two accumulators, 128 columns each).
 // What bounds it: the chain of 2 nl - 1 dependent steps of a tile (MMA, tensor memory to
-// registers, shared memory). A gradient of 4096 rows (18-128-128-128-2, to the host) takes 77 us,
+// registers, shared memory). A gradient of 4096 rows (18-128-128-128-2, to the host) takes 63 us,
 // and 215 us in twelve launches.
 #define FG_T 256
 static size_t fg_smem(int nl, int din0)
@@ -1145,7 +1145,7 @@ __global__ void __launch_bounds__(FG_T, 1) k_mlp_grad_tc(int n, const float* __r
 
 // the loss and the gradient of a batch into m->lossbuf and m->G: fused where a tile's operands of
 // all layers fit in shared memory (width 128, up to 32 inputs, 16 outputs and 3 hidden layers),
-// else layer by layer (4096 rows, 18-128-128-128-2, to the host: 77 us fused, 215 us layer by layer)
+// else layer by layer (4096 rows, 18-128-128-128-2, to the host: 63 us fused, 215 us layer by layer)
 static int mlp_loss_grad(pb_mlp* m, const float* X, const float* T, int n)
 {
     const size_t need = fg_smem(m->nl, m->din[0]), smem = 225 * 1024;  // one block per SM: it takes all tensor memory
