@@ -482,3 +482,48 @@ def test_several_vectors_add_tiles_in_fp64():
             assert np.all(np.abs(c - (a + b)) <= 5 * 2.0**-53 * big)
     finally:
         pb.pb_destroy(ctx)
+
+
+def test_scans_of_more_than_4096_tiles():
+    # 1,440,000 elements: the scan over three counts per element takes 4219 tiles, whose sums are scanned by
+    # themselves. It places the unordered touching pairs of the float-float integrals; the FP64 integrals
+    # do without, and both forms agree to 1e-11 (the bar of the float-float integrals)
+    n, w = 1200, 600
+    u, v = np.meshgrid(np.arange(n) * (2 * np.pi / n), np.arange(w) * (2 * np.pi / w), indexing="ij")
+    V = np.stack([(60 + 25 * np.cos(v)) * np.cos(u), (60 + 25 * np.cos(v)) * np.sin(u), 25 * np.sin(v)], -1).reshape(-1, 3)
+    i, j = np.meshgrid(np.arange(n), np.arange(w), indexing="ij")
+    a, b = (i * w + j).ravel(), (((i + 1) % n) * w + j).ravel()
+    c, d = (((i + 1) % n) * w + (j + 1) % w).ravel(), (i * w + (j + 1) % w).ravel()
+    T = np.concatenate([np.stack([a, b, c], 1), np.stack([a, c, d], 1)]).astype(np.int32)
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    x = _dev(inputs.random_density(m.nt, 7))
+    got = []
+    for singular in (pb.PB_SINGULAR_FF, pb.PB_SINGULAR_FP64):
+        ctx = _ctx(m, eta0=0.8, leaf_size=24, p=2, qs=2, precision=pb.PB_MIXED, precond=pb.PB_PRECOND_DIAG, singular=singular)
+        try:
+            assert pb.pb_get_tree_stats(ctx)["touching"] == 13 * m.nt  # six triangles at every vertex
+            y = torch.empty_like(x)
+            pb.pb_matvec_part(ctx, x, y, 1)
+            got.append(y.cpu().numpy())
+        finally:
+            pb.pb_destroy(ctx)
+    assert _rel(got[0], got[1]) < 1e-11
+
+
+@pytest.mark.parametrize("p", [9, 10])
+@pytest.mark.parametrize("prec,tol", [(pb.PB_FP64, 1e-13), (pb.PB_MIXED, 1e-6)])
+def test_several_vectors_at_high_orders(p, prec, tol):
+    # orders above 8 have more multi-indices than threads in the leaf moments: several vectors take the
+    # one-vector form of that kernel. Bars: the roundings of the working precision
+    V, T = inputs.perturbed_sphere(4, 9.0, 0.2, seed=5)
+    m = inputs.Mesh(V, T, np.zeros((1, 3)), np.ones(1))
+    ctx = _ctx(m, eta0=0.8, leaf_size=16, p=p, precision=prec, precond=pb.PB_PRECOND_DIAG)
+    try:
+        X = _dev(np.stack([inputs.random_density(m.nt, s) for s in range(5)]))
+        Y, y = torch.empty_like(X), torch.empty_like(X[0])
+        pb.pb_matvec_multi(ctx, X, Y)
+        for r in range(5):
+            pb.pb_matvec_part(ctx, X[r].contiguous(), y, 0)
+            assert _rel(Y[r].cpu().numpy(), y.cpu().numpy()) < tol
+    finally:
+        pb.pb_destroy(ctx)
