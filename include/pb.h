@@ -145,7 +145,9 @@ int pb_set_charges(pb_ctx* ctx, const double* q, int nc);
 /* Build everything that depends only on the geometry (Sections 2.3-2.6): element geometry,
  * Morton-ordered octree with shrink boxes, neighbour and interaction lists (def:eta),
  * singular Sauter-Schwab integrals of identical and adjacent triangle pairs, and the
- * preconditioner factors. Synchronises (list sizes are read back to size allocations). */
+ * preconditioner factors. Synchronises (list sizes are read back to size allocations).
+ * Beside what grows with the mesh, the FP64 near field keeps up to 256 MB of scratch (1 KB per
+ * pair of 32-element chunks of neighbouring leaves, at most 262,144 pairs at a time). */
 int pb_build_tree(pb_ctx* ctx);
 
 /* y = A x with A of def:linsys/eq_linsysEntry evaluated by the FMM (near field + Taylor
@@ -224,8 +226,9 @@ int pb_solvation_energy(pb_ctx* ctx, const double* x, double* E_kcal);
  * moments at the context's per-level orders (the product's P2M and MtM, run on x up to the
  * root), a leaf that fails is summed directly. O(N_c log N) instead of O(N_c N); the error
  * falls with the order and with theta (about 3e-7 relative at p = 8, theta = 0.5 on a
- * 1280-triangle sphere). x: device pointer; 0 < theta < 1; E_kcal: host pointer.
- * Synchronises. */
+ * 1280-triangle sphere). x: device pointer; 0 < theta < 1; E_kcal: host pointer. The energy
+ * repeats to the last bit. Takes about 4 KB of device memory per charge (for up to 16,384 charges
+ * at a time) for the time of the call, or does without at a lower speed. Synchronises. */
 int pb_solvation_energy_treecode(pb_ctx* ctx, const double* x, double theta, double* E_kcal);
 
 /* Tree statistics after pb_build_tree. out: host pointer. Synchronises. */
@@ -254,8 +257,8 @@ int pb_matvec_part(pb_ctx* ctx, const double* x, double* y, int which);
 #define PB_MAX_RHS 64
 
 #define PB_TIMING_SLOTS 13
-#define PB_T_NEAR 0       /* near-field kernel (one-point rule + mass terms) */
-#define PB_T_CORR 1       /* Sauter-Schwab corrections of touching pairs */
+#define PB_T_NEAR 0       /* near field */
+#define PB_T_CORR 1       /* Sauter-Schwab corrections of touching pairs and the end of a product */
 #define PB_T_UP 2         /* leaf moments and MtM */
 #define PB_T_M2L 3        /* MtL on all levels */
 #define PB_T_DOWN 4       /* LtL and LtP */
